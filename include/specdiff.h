@@ -381,7 +381,8 @@ int sdv_sampler_end(int B, int L, int64_t d, void *workspace, size_t workspace_b
 /*
  * sdv_em_sample - the plain (non-speculative) Euler-Maruyama chain, Y_{k+1} =
  * m^q_k(Y_k) + sigma_k G_k for k = 0 .. K-1 from Y_0 (stream 5), G_k from stream 6 with
- * sub-counter k; y_out [B, d] fp32 out.  K kernel launches on `stream`.
+ * sub-counter k; y_out [B, d] fp32 out.  One kernel on `stream` runs all K
+ * steps (two launches for d > 1024).
  */
 int sdv_em_sample(int B, int64_t d, const float *means, const float *log_weights, int C,
                   float comp_var, int K, float churn, float beta_min, float beta_max,

@@ -666,15 +666,166 @@ k_sampler_init(int B, int L, int64_t d, int K, uint64_t seed, float* y, int32_t*
   }
 }
 
-// One plain Euler-Maruyama step for every chain, in place: y <- m^q_k(y) + sigma_k G_k;
-// one warp per chain.
+// The plain Euler-Maruyama chain for rows of up to 128 NG elements: a team of T warps runs
+// a chain's K steps with the state in registers (every warp holds all of it, lane l the
+// groups l, l + 32, ...) and the means in shared memory, one copy per CTA.  Per step the
+// warps share out the components (squared distances, pass 1), then the groups (score,
+// mean and noise, pass 2), and exchange the logits and the new state through shared
+// memory.  The sums have the order of gmm_rows_warp, so that both give the same states.
+// It is bound by instruction issue (of about 315 instructions per group of four and step,
+// 190 draw its noise); one launch per step with the state in HBM took 13.1 us a step at
+// B = 1024, d = 1024, C = 8, this kernel 4.7 us with T = 4 (T = 2: 5.5, too few warps; 8:
+// 5.4, seven eighths of the softmax repeated and two waves of CTAs).
+constexpr int kEmMaxTeams = 7;   // chains per CTA: 152 SMs x 7 hold 1024 chains in one wave
+
+template <int MAXC, int NG, int T>
+__global__ void __launch_bounds__(32 * T * (T == 8 ? 1 : kEmMaxTeams))
+k_em_chain(float* __restrict__ y, int B, int64_t d, Sched S, Gmm G, uint64_t seed) {
+  extern __shared__ float4 em_s[];
+  constexpr int GP = 32 * NG;            // groups of a padded row
+  constexpr int CPW = MAXC / T;          // components per warp
+  const unsigned FULL = 0xffffffffu;
+  const int C = G.C;
+  const int dn = (int)d;
+  const int teams = blockDim.x / (32 * T);
+  const int team = threadIdx.x / (32 * T), lane = threadIdx.x & 31;
+  const int tw = (threadIdx.x >> 5) - team * T;
+  float4* mu_s = em_s;                                           // [C][GP], zero past d
+  float4* z_s = em_s + (size_t)C * GP + (size_t)team * GP;       // [teams][GP]
+  float* lg_s = reinterpret_cast<float*>(em_s + (size_t)(C + teams) * GP) + team * MAXC;
+  for (int i = threadIdx.x; i < C * GP * 4; i += blockDim.x) {
+    const int c = i / (GP * 4), e = i - c * (GP * 4);
+    reinterpret_cast<float*>(mu_s)[i] = e < dn ? __ldg(G.means + (int64_t)c * d + e) : 0.f;
+  }
+  __syncthreads();
+  const int b = blockIdx.x * teams + team;
+  if (b >= B) return;                    // the whole team
+  auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(32 * T) : "memory"); };
+  // elements past d hold 0 (they then add exactly nothing to the distances)
+  auto masked = [&](float4 v, int gi) {
+    const int e = dn - 4 * gi;
+    if (e < 4) {
+      if (e < 1) v.x = 0.f;
+      if (e < 2) v.y = 0.f;
+      if (e < 3) v.z = 0.f;
+      v.w = 0.f;
+    }
+    return v;
+  };
+  float4 z[NG];
+  for (int i = tw; i < NG; i += T) {
+    const int gi = lane + 32 * i;
+    z_s[gi] = masked(normals4(seed, (uint32_t)b, (uint32_t)gi, kStreamInit, 0u), gi);
+  }
+  team_sync();
+#pragma unroll
+  for (int i = 0; i < NG; ++i) z[i] = z_s[lane + 32 * i];
+  const float cst = 0.5f * (1.0f + S.churn * S.churn);
+  float sab_l = 0.f, iv_l = 0.f, be_l = 0.f, sg_l = 0.f;   // schedule of step (k & ~31) + lane
+  for (int k = 0; k < S.K; ++k) {
+    if ((k & 31) == 0) {
+      const int kl = min(k + lane, S.K);
+      const float tf = S.tfwd(kl);
+      const float ab = S.abar(tf);
+      sab_l = sqrtf(ab);
+      const float v = ab * G.comp_var + 1.0f - ab;
+      iv_l = 1.0f / v;
+      be_l = S.beta(tf);
+      sg_l = S.sigma(kl);
+    }
+    const float sab = __shfl_sync(FULL, sab_l, k & 31), inv_v = __shfl_sync(FULL, iv_l, k & 31);
+    const float be = __shfl_sync(FULL, be_l, k & 31), sg = __shfl_sync(FULL, sg_l, k & 31);
+    // pass 1: squared distances to this warp's scaled centres
+    float acc[CPW];
+#pragma unroll
+    for (int m = 0; m < CPW; ++m) acc[m] = 0.f;
+#pragma unroll
+    for (int i = 0; i < NG; ++i) {
+      const float zf[4] = {z[i].x, z[i].y, z[i].z, z[i].w};
+#pragma unroll
+      for (int m = 0; m < CPW; ++m) {
+        const int c = tw * CPW + m;
+        if (c < C) {
+          const float4 t = mu_s[c * GP + lane + 32 * i];
+          const float mf[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const float df = zf[e] - sab * mf[e];
+            acc[m] = fmaf(df, df, acc[m]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int m = 0; m < CPW; ++m) {
+      const int c = tw * CPW + m;
+      float a = acc[m];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(FULL, a, o);
+      if (lane == 0) lg_s[c] = (c < C) ? __ldg(G.log_w + c) - 0.5f * a * inv_v : -INFINITY;
+    }
+    team_sync();
+    float r[MAXC];
+    float mx = -INFINITY;
+#pragma unroll
+    for (int c = 0; c < MAXC; ++c) {
+      r[c] = lg_s[c];
+      mx = fmaxf(mx, r[c]);
+    }
+    float den = 0.f;
+#pragma unroll
+    for (int c = 0; c < MAXC; ++c) {
+      r[c] = (c < C) ? expf(r[c] - mx) : 0.f;
+      den += r[c];
+    }
+    const float w_sc = sab / den;
+    // pass 2: this warp's groups of the new state
+#pragma unroll
+    for (int ii = 0; ii < (NG + T - 1) / T; ++ii) {
+      const int i = tw + ii * T;
+      if (NG % T != 0 && i >= NG) break;   // warp-uniform
+      const int gi = lane + 32 * i;
+      const float4 n4 = normals4(seed, (uint32_t)b, (uint32_t)gi, kStreamEM, (uint32_t)k);
+      const float G4[4] = {n4.x, n4.y, n4.z, n4.w};
+      const float4 zo = z_s[gi];
+      const float zf[4] = {zo.x, zo.y, zo.z, zo.w};
+      float wsum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int c = 0; c < MAXC; ++c) {
+        if (c < C) {
+          const float4 t = mu_s[c * GP + gi];
+          const float mf[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) wsum[e] = fmaf(r[c], mf[e], wsum[e]);
+        }
+      }
+      float m[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float sc = (w_sc * wsum[e] - zf[e]) * inv_v;
+        m[e] = zf[e] + S.delta * (0.5f * be * zf[e] + cst * be * sc) + sg * G4[e];
+      }
+      z_s[gi] = masked(make_float4(m[0], m[1], m[2], m[3]), gi);
+    }
+    team_sync();
+#pragma unroll
+    for (int i = 0; i < NG; ++i) z[i] = z_s[lane + 32 * i];
+  }
+  float* row = y + (int64_t)b * d;
+  const float* zr = reinterpret_cast<const float*>(z_s);
+  for (int e = tw * 32 + lane; e < dn; e += 32 * T) row[e] = zr[e];
+}
+
+// The plain Euler-Maruyama chain for longer rows: one warp runs a chain's K steps, the
+// state in its row of y (each group read and written by one lane only).
 template <int MAXC, bool VEC>
 __global__ void __launch_bounds__(kGmmThreads)
-k_em_step(float* y, int B, int64_t d, int k, Sched S, Gmm G, bool use_smem, uint64_t seed) {
+k_em_rows(float* y, int B, int64_t d, Sched S, Gmm G, bool use_smem, uint64_t seed) {
   const float* mu = stage_means(G, d, use_smem);
-  const int warp = threadIdx.x >> 5;
-  for (int b = blockIdx.x * kGmmWarps + warp; b < B; b += gridDim.x * kGmmWarps) {
-    float* row = y + (int64_t)b * d;
+  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (b >= B) return;
+  float* row = y + (int64_t)b * d;
+  for (int k = 0; k < S.K; ++k) {
     const GmmRow R[1] = {{row, row, nullptr, k, (uint32_t)b, S.sigma(k)}};
     gmm_rows_warp<MAXC, VEC, 1>(R, 1, d, S, G, mu, seed, kStreamEM);
   }
@@ -693,7 +844,7 @@ template <int MAXC, bool VEC>
 static void gmm_set_smem(size_t bytes) {
   cudaFuncSetAttribute(k_gmm_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
   cudaFuncSetAttribute(k_round_target<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_em_step<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  cudaFuncSetAttribute(k_em_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // rows_aligned: every state / output row the kernel touches starts on a 16-byte boundary
@@ -761,6 +912,39 @@ static int launch_check() {
     return SDV_ECUDA;
   }
   return SDV_OK;
+}
+
+// The plain chain of rows of up to 1024 elements: teams of T warps, chains dealt evenly to
+// the SMs, at most kEmMaxTeams to a CTA.
+template <int MAXC, int NG, int T>
+static int launch_em_t(int B, int64_t d, const Sched& S, const Gmm& G, uint64_t seed, float* y, cudaStream_t s) {
+  const int sms = sm_count();
+  const int teams = T == 8 ? 1 : std::min(kEmMaxTeams, std::max(1, (B + sms - 1) / sms));
+  const size_t smem = sizeof(float4) * (size_t)(G.C + teams) * 32 * NG + sizeof(float) * (size_t)teams * MAXC;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_em_chain<MAXC, NG, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) {
+      set_last_cuda_error((int)e);
+      cudaGetLastError();
+      return SDV_ECUDA;
+    }
+  }
+  k_em_chain<MAXC, NG, T><<<(unsigned)((B + teams - 1) / teams), 32 * T * teams, smem, s>>>(y, B, d, S, G, seed);
+  return launch_check();
+}
+
+template <int MAXC>
+static int launch_em(int B, int64_t d, const Sched& S, const Gmm& G, uint64_t seed, float* y, cudaStream_t s) {
+  // eight warps to a chain while every chain has an SM to itself, else four
+  const bool wide = B <= sm_count();
+#define SDV_EM(NG)                                                    \
+  return wide ? launch_em_t<MAXC, NG, 8>(B, d, S, G, seed, y, s)       \
+              : launch_em_t<MAXC, NG, 4>(B, d, S, G, seed, y, s)
+  if (d <= 128) { SDV_EM(1); }
+  if (d <= 256) { SDV_EM(2); }
+  if (d <= 512) { SDV_EM(4); }
+  SDV_EM(8);
+#undef SDV_EM
 }
 
 static bool valid_sched(int K, float churn, float bmin, float bmax, float tfl) {
@@ -1092,6 +1276,9 @@ int sdv_em_sample(int B, int64_t d, const float* means, const float* log_weights
   cudaStream_t s = (cudaStream_t)stream;
   const Sched S = make_sched(K, churn, beta_min, beta_max, t_floor);
   const Gmm G{means, log_weights, C, comp_var};
+  // rows of up to 1024 elements fit the registers of a team; longer ones stay in memory
+  if (d <= 1024)
+    return C <= 8 ? launch_em<8>(B, d, S, G, seed, y_out, s) : launch_em<16>(B, d, S, G, seed, y_out, s);
   const int64_t ng = (int64_t)B * ((d + 3) / 4);
   // the initial state only needs y; the bookkeeping arrays of the init kernel are not used
   k_sampler_init<<<(unsigned)((ng + 255) / 256), 256, 0, s>>>(B, 1, d, K, seed, y_out, nullptr, nullptr,
@@ -1099,11 +1286,8 @@ int sdv_em_sample(int B, int64_t d, const float* means, const float* log_weights
   int rc = launch_check();
   if (rc != SDV_OK) return rc;
   const GmmLaunch gl = gmm_launch(C, d, means, reinterpret_cast<uintptr_t>(y_out) % 16 == 0);
-  for (int k = 0; k < K; ++k) {
-    SDV_GMM_DISPATCH(gl, k_em_step, rows_grid(B), s, y_out, B, d, k, S, G, gl.smem, seed);
-    if ((rc = launch_check()) != SDV_OK) return rc;
-  }
-  return SDV_OK;
+  SDV_GMM_DISPATCH(gl, k_em_rows, rows_grid(B), s, y_out, B, d, S, G, gl.smem, seed);
+  return launch_check();
 }
 
 }  // extern "C"

@@ -143,6 +143,25 @@ def test_em_chain_matches_oracle(api, K, Bn, d, chains):
     assert err <= tol
 
 
+# Edges of the EM kernels: rows of one group, around 128 NG elements (registers of a team)
+# and past 1024 (rows in memory), odd tails, more than 8 components; one chain, one chain
+# per SM and one more (teams of eight and of four warps), and more chains than one wave.
+@pytest.mark.parametrize("Bn,d,C", [(1, 1, 1), (2, 3, 8), (152, 128, 8), (153, 129, 9), (1070, 127, 2),
+                                    (1070, 1024, 8), (5, 513, 16), (160, 1023, 16), (9, 1025, 12), (3, 1028, 8)])
+def test_em_kernel_edges(api, Bn, d, C):
+    # K = 200 steps as in test_em_chain_matches_oracle, whose bound holds where a step's
+    # Jacobian is close to 1: 1 + delta beta / 2 is at most 1.05 here (2.7 for K = 6, where
+    # six steps grow a rounding error a hundredfold and 1e-5 is no bound)
+    K = 200
+    gmm = _gmm(C, d, 15)
+    sch = OS.VPSchedule(K, 0.5)
+    ch = np.unique(np.linspace(0, Bn - 1, 20).astype(int))
+    y = api.em_sample(Bn, _target(api, gmm, K, 0.5), 21).cpu().numpy()
+    yo = OS.em_sample(Bn, d, gmm, sch, 21, chains=ch)
+    assert np.isfinite(y).all()
+    assert np.abs(y[ch] - yo).max() <= max(1e-5, 4.0 * math.sqrt(K) * 2.0 * 2.0 ** -24 * np.abs(yo).max())
+
+
 def _first_rounds(api, mode, drafter, d, C, Bn=192, L=4, K=40, gmm=None, chains=None, churn=0.5,
                   seed=123):
     """Rounds 1..3 of the GPU sampler (all Bn chains) against the oracle on `chains`: k
