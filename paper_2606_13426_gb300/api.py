@@ -20,12 +20,13 @@ def _ptr(t):
 
 
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    # the handle alone: building a Stream object takes longer than a small call's launch
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _need_cuda(*ts):
     for t in ts:
-        if t is not None and (not t.is_cuda or not t.is_contiguous()):
+        if t is not None and not (t.is_cuda and t.is_contiguous()):
             raise ValueError("libspecdiff needs contiguous CUDA tensors")
 
 
@@ -86,13 +87,14 @@ def verify(x_draft, mu_target, mu_draft, sigma, seed, mode="block", *, L_eff=Non
         aux = torch.empty(Bn, 4, dtype=torch.float32, device=dev) if aux is None else aux
     if workspace is None:
         workspace = make_workspace(Bn, L, d, dt, dev)
-    fn = B.sdv_verify_pipelined if pipelined else B.sdv_verify_ex
-    fn(_ptr(x_draft), _ptr(mu_target), _ptr(mu_draft), _ptr(sigma), sstride,
-       Bn, L, d, _DTYPES[dt], int(seed) & 0xFFFFFFFFFFFFFFFF, _MODES[mode],
-       _ptr(L_eff), _ptr(mu_target_bonus), _ptr(sigma_bonus),
-       _RESIDUALS[residual], float(omega),
-       _ptr(acc), _ptr(y), _ptr(lr), _ptr(dn), _ptr(st), _ptr(aux),
-       _ptr(workspace), workspace.numel(), _stream())
+    # straight to the C entry point (the binding's function of that name has the same arguments)
+    B._call("sdv_verify_pipelined" if pipelined else "sdv_verify_ex",
+            x_draft.data_ptr(), mu_target.data_ptr(), mu_draft.data_ptr(), sigma.data_ptr(), sstride,
+            Bn, L, d, _DTYPES[dt], int(seed) & 0xFFFFFFFFFFFFFFFF, _MODES[mode],
+            _ptr(L_eff), _ptr(mu_target_bonus), _ptr(sigma_bonus),
+            _RESIDUALS[residual], float(omega),
+            acc.data_ptr(), y.data_ptr(), _ptr(lr), _ptr(dn), st.data_ptr(), _ptr(aux),
+            workspace.data_ptr(), workspace.numel(), _stream())
     res = dict(accepted_len=acc, y=y, status=st)
     if with_ratios:
         res.update(log_ratio=lr, delta_norm=dn)

@@ -6,10 +6,12 @@ raises ``SDVError`` on a non-zero return code.  The library is loaded on first
 use; a missing library raises instead of falling back to anything else.
 """
 import ctypes
+import functools
+import importlib.util
 import os
 import threading
 
-from .buildlib import lib_path
+from .buildlib import lib_path, pycall_path
 
 SDV_OK = 0
 SDV_EINVAL = -1
@@ -79,6 +81,7 @@ SIGNATURES = {
 }
 
 _lib = None
+_fns = {}                     # name -> callable with the C entry point's arguments
 _lock = threading.Lock()
 
 
@@ -106,8 +109,24 @@ def load(path=None):
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+            _fns[name] = fn
+        _bind_native(lib)
         _lib = lib
         return lib
+
+
+def _bind_native(lib):
+    """The calls of a serving loop through the compiled module (ctypes takes 4-5 us to convert
+    their 25 arguments); without it (built where Python's headers are missing) ctypes serves."""
+    path = pycall_path()
+    if not os.path.exists(path):
+        return
+    spec = importlib.util.spec_from_file_location("_sdvcall", path)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    for name, fn in (("sdv_verify_ex", mod.verify), ("sdv_verify_pipelined", mod.verify),
+                     ("sdv_log_ratios", mod.ratios)):
+        _fns[name] = functools.partial(fn, ctypes.cast(getattr(lib, name), ctypes.c_void_p).value)
 
 
 def strerror(code):
@@ -117,10 +136,14 @@ def strerror(code):
 
 
 def _call(name, *args):
-    lib = load()
-    rc = getattr(lib, name)(*args)
+    if _lib is None:              # loaded once, under the lock
+        load()
+    try:
+        rc = _fns[name](*args)
+    except TypeError:             # not a plain argument list: ctypes converts or refuses it
+        rc = getattr(_lib, name)(*args)
     if rc != SDV_OK:
-        raise SDVError(name, rc, lib.sdv_last_cuda_error() if rc == SDV_ECUDA else 0)
+        raise SDVError(name, rc, _lib.sdv_last_cuda_error() if rc == SDV_ECUDA else 0)
     return rc
 
 

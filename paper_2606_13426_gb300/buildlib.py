@@ -1,13 +1,15 @@
 """Build libspecdiff.so (the C-ABI library) for sm_103a with nvcc.
 
 Sources are compiled in parallel, one nvcc process per translation unit, and
-linked into ``paper_2606_13426_gb300/lib/libspecdiff.so``.  A rebuild happens only
+linked into ``paper_2606_13426_gb300/lib/libspecdiff.so``; the CPython module of the
+binding's frequent calls goes beside it.  A rebuild happens only
 when a source or header is newer than the library (or ``force=True``).
 """
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -26,6 +28,25 @@ def lib_path():
     return os.path.join(LIBDIR, LIBNAME)
 
 
+def pycall_path():
+    return os.path.join(LIBDIR, "_sdvcall.so")
+
+
+def _build_pycall():
+    """The CPython module of sdv_pycall.c; left out where Python's headers are missing (the
+    binding then calls through ctypes)."""
+    inc = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(inc, "Python.h")):
+        return
+    out = pycall_path()
+    cmd = [os.environ.get("CC") or shutil.which("gcc") or "cc", "-O2", "-shared", "-fPIC", "-I" + INCLUDE, "-I" + inc,
+           os.path.join(CSRC, "sdv_pycall.c"), "-o", out + ".tmp"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("compiling sdv_pycall.c failed:\n%s\n%s" % (" ".join(cmd), r.stderr))
+    os.replace(out + ".tmp", out)
+
+
 def _nvcc():
     for cand in (os.environ.get("NVCC"), shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
         if cand and os.path.exists(cand):
@@ -38,7 +59,7 @@ def _sources():
 
 
 def _deps():
-    deps = _sources()
+    deps = _sources() + [os.path.join(CSRC, "sdv_pycall.c")]
     for d in (CSRC, INCLUDE):
         deps += [os.path.join(d, f) for f in os.listdir(d) if f.endswith((".h", ".cuh"))]
     return deps
@@ -75,6 +96,7 @@ def build(force=False, verbose=False):
     srcs = _sources()
     with ThreadPoolExecutor(max_workers=max(1, len(srcs))) as ex:
         objs = list(ex.map(compile_one, srcs))
+    _build_pycall()
     tmp = out + ".tmp"
     cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs
     r = subprocess.run(cmd, capture_output=True, text=True)
