@@ -83,9 +83,10 @@ def peaks():
 
 
 def kernel_sources_digest():
-    """sha256 over the sources that define the fused verify kernel (in a fixed order)."""
+    """sha256 over the sources that define the verify kernels (in a fixed order)."""
     h = hashlib.sha256()
-    for f in ("sdv_verify.cu", "sdv_device.cuh", "sdv_host.h"):
+    for f in ("sdv_verify.cu", "sdv_device.cuh", "sdv_host.h", "sdv_scan.cuh", "sdv_tiles.cuh", "sdv_finish.cuh",
+              "sdv_chain.cuh"):
         with open(os.path.join(ROOT, "paper_2606_13426_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -151,15 +152,14 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# Rows of more than this many groups of four elements get their residual from two
-# extra kernels (the library's kFusedMaxGroups and kFinishMaxGroups); pipelined calls
-# keep rows of up to PIPE_MAX_GROUPS in k_finish (kPipeMaxGroups).
+# The phases of a call by its sizes: rows of more than this many groups of four elements have
+# their residual's sum and write counted apart; pipelined calls finish rows of up to
+# PIPE_MAX_GROUPS in k_finish (the library's kPipeMaxGroups).
 FUSED_MAX_GROUPS = 1024
 FINISH_MAX_GROUPS = 1024
 PIPE_MAX_GROUPS = 4096
 
-# From this many chains on, the library streams the tiles with k_tiles and finishes
-# every chain with one warp of k_finish (the library's kManyChainMin).
+# From this many chains on, a call is counted as streaming and finishing.
 MANY_CHAIN_MIN = 512
 
 
@@ -180,7 +180,7 @@ def wide_finish(B, d, pipelined=False):
     return FINISH_MAX_GROUPS < ng <= PIPE_MAX_GROUPS and (pipelined or not many_chains(B))
 
 
-# Plain calls with fewer chains run the fused kernel (the library's kFusedMaxChains).
+# Plain calls with fewer chains are counted as one phase.
 FUSED_MAX_CHAINS = 64
 
 
@@ -189,25 +189,31 @@ def _two_kernels(B, d, pipelined):
 
 
 def long_rows(d, B=0, pipelined=False):
-    """Rows whose residual two extra kernels write (longer than the finishing CTA's noise
-    cache: the fused kernel's, or k_finish's)."""
+    """Rows whose residual counts as two more phases (longer than one finishing CTA's noise
+    cache)."""
     if wide_finish(B, d, pipelined):
         return False
     return (d + 3) // 4 > (FINISH_MAX_GROUPS if _two_kernels(B, d, pipelined) else FUSED_MAX_GROUPS)
 
 
 def launches_per_step(B, d, pipelined=False):
-    """Kernels one verification call launches: the fused verify kernel, or k_tiles and
-    k_finish (many chains, a pipelined call, or rows of 1025-4096 groups), plus the
-    residual dot / write kernels for long rows."""
+    """Phases of a verification call by its sizes: the whole call, or streaming and finishing
+    (many chains, a pipelined call, or rows of 1025-4096 groups), plus the residual's sum and
+    write for long rows.  Several may share a kernel: kernels_of_step lists the launches."""
     return (2 if _two_kernels(B, d, pipelined) else 1) + (2 if long_rows(d, B, pipelined) else 0)
 
 
-def kernels_of_step(B, d, pipelined=False):
-    names = ["k_tiles", "k_finish"] if _two_kernels(B, d, pipelined) else ["k_verify"]
-    if long_rows(d, B, pipelined):
-        names += ["k_resid_dot", "k_resid_write"]
-    return names
+def kernels_of_step(B, d, pipelined=False, L=8, dt_name="f32"):
+    """Kernels one verification call launches, in order (sizes of the library's routing rule,
+    152 SMs; without its limits on clusters of CTAs and on shared memory)."""
+    if not pipelined and B <= 304:
+        es = 2 if dt_name == "bf16" else 4
+        vecs = -(-d * es // 16)
+        tiles = L * -(-vecs // (256 * max(1, min(2 if es == 2 else 4, -(-vecs // 256)))))
+        cl = max(1, min(8, tiles, 304 // B))
+        if 10 * B * cl >= 13 * 152 or 3 * L * d * es // cl <= 256 * 1024:
+            return ["k_chain"]
+    return ["k_tiles", "k_finish" if (d + 3) // 4 <= PIPE_MAX_GROUPS else "k_finish_long"]
 
 
 def call_bytes(B, L, d, dtype):
@@ -579,10 +585,7 @@ def measure_verify(api, name, Bn, mode, steps, warmup, dev, rank, pg=None, clock
         value_per_rank=Bn * L / (ms_step * 1e-3), taus=taus, clocks=clk, host0=host0,
         roofline={"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                   "frac": achieved / hbm_peak, "peak_kind": peak_kind,
-                  "kernel": ("k_verify (fused: log-ratio pass, acceptance, U-draw, residual write)"
-                             if launches_per_step(Bn, d, pipelined) == 1 else
-                             "whole call (%d kernels: %s)" % (launches_per_step(Bn, d, pipelined),
-                                                             ", ".join(kernels_of_step(Bn, d, pipelined)))),
+                  "kernel": "whole call (%s)" % ", ".join(kernels_of_step(Bn, d, pipelined, L, dt_name)),
                   "duration": "per-call period of 200 back-to-back calls in one CUDA graph "
                               "(events at its two ends only)",
                   "duration_us": 1e3 * ms_call, "algorithmic_bytes": nbytes,
@@ -708,7 +711,7 @@ def main():
                 "hbm_gbs_step": r["roofline"]["algorithmic_bytes"] / (r["ms_step"] * 1e-3) / 1e9,
                 "roofline": r["roofline"], "mean_tau_block": r["taus"]["block"],
                 "mean_tau_sample": r["taus"]["sample"],
-                "gpu_launches": launches_per_step(c["B"], c["d"], pipelined) * args.steps}
+                "gpu_launches": len(kernels_of_step(c["B"], c["d"], pipelined, c["L"], c["dtype"])) * args.steps}
         subs["sampler"] = sampler_summary(api, dev)
 
     e2e_steps = max(20, min(400, args.steps))
@@ -739,7 +742,7 @@ def main():
                 "d2h_bytes_per_step": d2h,
                 "api": "api.HostStream (pinned [3,B,L,d] window in, accepted_len and y out, "
                        "copy of step i+1 overlapping step i)"},
-        "gpu_launches": launches_per_step(Bn, d, pipelined) * args.steps,
+        "gpu_launches": len(kernels_of_step(Bn, d, pipelined, L, dt_name)) * args.steps,
         "clocks": head["clocks"],
         "workloads": subs,
     }

@@ -159,8 +159,8 @@ int sdv_verify_ex(const void *x_draft, const void *mu_target, const void *mu_dra
  * rule, U-draw and residual) overlaps the next call's read of its window.  The
  * verification itself is the same (Algorithms token-/block-verification,
  * decomposition-res, u-sample): log ratios, accepted lengths and status equal
- * sdv_verify_ex's bit for bit; U and y agree within the library's accuracy (rows of
- * up to 4096 elements finish in a 64-thread CTA with the one-warp U-sampler).
+ * sdv_verify_ex's bit for bit; U and y agree within the library's accuracy (other
+ * threads add up e^T G).
  * Precondition (the caller's promise; nothing checks it): the window (x_draft,
  * mu_target, mu_draft, sigma, L_eff, mu_target_bonus, sigma_bonus) is not written by
  * earlier work on `stream` that may still be running: the previous kernel, and the
@@ -171,8 +171,7 @@ int sdv_verify_ex(const void *x_draft, const void *mu_target, const void *mu_dra
  * waits for the previous kernel), and the finishing kernel waits for the whole stream
  * of its call when it reads a partial without its call's tag.
  * Outputs are written only after the previous call on `stream` has written its own,
- * so consecutive calls may share output buffers.  Rows longer than 16384 elements
- * add two residual kernels, which overlap the next call's stream too.  Same
+ * so consecutive calls may share output buffers.  Same
  * arguments, return codes and ownership as sdv_verify_ex; the workspace must not be
  * shared with calls on other streams.
  */
@@ -393,10 +392,8 @@ int sdv_em_sample(int B, int64_t d, const float *means, const float *log_weights
  * sdv_verify_ex calls made on this host thread record CUDA events on their
  * stream into a ring of `slots` entries (one call in `every`, see
  * sdv_timing_stride; every call by default): before the first kernel of the
- * call, after it (the fused verify kernel; with B >= 512 chains the streaming
- * kernel of the many-chain path), and after the kernels that follow it (the
- * many-chain finishing kernel, and the separate residual kernels used for rows
- * longer than 4096 elements).  Calls made by sdv_sampler_run / sdv_sampler_round
+ * call, after it (the whole call where one kernel runs it, else the streaming kernel),
+ * and after the finishing kernel that follows it, if any.  Calls made by sdv_sampler_run / sdv_sampler_round
  * are not recorded.  The records are ordinary stream work, so they are captured into
  * a CUDA graph like the kernels (an event record costs a few microseconds of
  * graph time, hence the stride).  The events are created here (host objects; no
@@ -413,11 +410,9 @@ int sdv_timing_stride(int every);
 /*
  * Waits for the events of the last `n_calls` recorded calls (1 <= n_calls <=
  * slots) and writes their summed phase times in milliseconds:
- * ms3[0] the first kernel (the fused verify kernel: log-ratio pass, acceptance,
- * U-draw and, for rows up to 4096 elements, the residual write; or, with B >= 512,
- * the many-chain streaming kernel), ms3[1] the kernels after it (the many-chain
- * finishing kernel and the long-row residual kernels; the time of the event
- * records alone when there are none), ms3[2] reserved (0).  SDV_EINVAL if timing
+ * ms3[0] the first kernel (the whole call, or the streaming kernel), ms3[1] the finishing
+ * kernel (the time of the event records alone when there is none), ms3[2] reserved (0).
+ * SDV_EINVAL if timing
  * is off or fewer calls were recorded.
  */
 int sdv_timing_read(int n_calls, float *ms3);

@@ -8,52 +8,34 @@
 
 namespace sdv {
 
-// Fused verify kernel: threads per CTA and 16-byte vectors per thread per tensor per sweep.
+// Streaming kernels: threads per CTA and 16-byte vectors per thread per tensor of a tile.
 constexpr int kK1Threads = 256;
 constexpr int kK1Vpt = 4;
-// Resident CTAs per SM the fused kernel is built for (its register budget): the
-// chain-finishing code needs more than the streaming loop.
-constexpr int kK1MinBlocks = 4;
-// Many-chain path (B >= kManyChainMin): resident CTAs per SM of the streaming
-// kernel k_tiles (its register budget: 3 x vpt 16-byte buffers per thread), and
-// the finishing kernel k_finish: threads per chain and groups of four elements per
-// thread per residual sweep.
+// With this many chains of at most kFinishManyMaxGroups groups of 4 elements, k_finish takes
+// fewer threads each.
 constexpr int kManyChainMin = 512;
-// Plain calls with fewer chains than this run the fused kernel (one launch; its
-// staggered per-chain finishing wins for small batches); from this many on, k_tiles +
-// k_finish (measured per call, pixel rows: B = 16 18.5 against 22.5 us, B = 64 24.9
-// against 24.3, B = 256 38.2 against 34.8 in block mode).
-constexpr int kFusedMaxChains = 64;
-// Three vectors per thread fit 48 registers, so that four k_tiles CTAs still leave
-// room for two 64-thread k_finish CTAs of the previous pipelined call on the same SM
-// (pipelined pixel rows 16.4 -> 16.3 us per call in block mode, 16.2 -> 15.7 in sample).
+constexpr int64_t kFinishManyMaxGroups = 256;
+// Resident k_tiles CTAs per SM (its register budget).  Three vectors per thread fit 48
+// registers, so that the stream still finds room beside the previous pipelined call's
+// k_finish CTAs.
 constexpr int tile_min_blocks(int vpt) { return vpt <= 1 ? 8 : (vpt == 2 ? 6 : (vpt == 3 ? 5 : 4)); }
-constexpr int kFinishThreads = 64;
+constexpr int kFinishThreads = 128;
+constexpr int kFinishThreadsMany = 64;
 constexpr int kFinishWideThreads = 256;
-constexpr int kFinishResidUnroll = 4;
+// Rows of up to kElementMax elements have at most kElementsPerThread for a thread.
+constexpr int kElementsPerThread = 4;
+constexpr int64_t kElementMax = kElementsPerThread * kK1Threads;
 // Stand-alone acceptance scan: one warp per chain.
 constexpr int kK2Threads = 128;
-// Long-row residual kernels: threads per CTA, and the elements of the rejected row
-// per CTA, chosen per call between kK4MinChunk and kK4MaxChunk so that the grid is
-// about kK4TargetCtas CTAs (short kernels want many CTAs; long rows want fewer,
-// longer ones).
-constexpr int kK4Threads = 256;
-constexpr int64_t kK4MinChunk = 1024;
-constexpr int64_t kK4MaxChunk = 4096;
-constexpr int64_t kK4TargetCtas = 1024;
-// Pipelined calls: at most this many CTAs per long-row residual kernel (they sit
-// resident, waiting for the chain states, while the next call streams).
-constexpr int64_t kK4PipeCtas = 128;
-// Rows of up to kFusedMaxGroups groups of 4 elements are written by the CTA that
-// finishes the chain inside the fused kernel, kFinishMaxGroups by k_finish on the
-// many-chain path, and kPipeMaxGroups by k_finish on the pipelined path (in each case
-// the residual's noise cached in dynamic shared memory: 16 KB, or up to 64 KB);
-// longer rows by k_resid_dot/_write.  The fused kernel's residual sweeps take
-// kFusedResidUnroll groups per thread, their loads issued together.
-constexpr int64_t kFusedMaxGroups = 1024;
+// Rows of up to kFinishMaxGroups groups of 4 elements are finished by k_finish's
+// kFinishThreads, up to kPipeMaxGroups by kFinishWideThreads (the residual's noise cached in
+// dynamic shared memory, 16 KB or up to 64 KB); longer rows by k_finish_long.
 constexpr int64_t kFinishMaxGroups = 1024;
 constexpr int64_t kPipeMaxGroups = 4096;
-constexpr int kFusedResidUnroll = 3;
+
+// How the kernels read the rows of a window: element by element, as whole aligned 16-byte
+// vectors, or as vectors over rows that start anywhere within one (arrays 16-byte aligned).
+enum : int { kRowsElement = 0, kRowsAligned = 1, kRowsUnaligned = 2 };
 
 enum : int32_t {
   kKindInactive = 0,
@@ -80,7 +62,6 @@ struct ChainState {
 };
 
 struct ScanArgs {
-  const float2* part;     // fused kernel: [B, L, C] (S1, S2) per tile
   const uint64_t* tpart;  // k_tiles: [B, L, C] pairs of words (S1 | tag << 32, S2 | tag << 32)
   uint32_t* consumed;     // [B, L, C] beside tpart: the tag of the partial last read from each slot
   uint32_t tag;           // this call's tag of its k_tiles partials (never 0)
@@ -109,16 +90,29 @@ struct ScanArgs {
   bool draw_u;  // draw the residual U (the whole verify step) or stop at tau
 };
 
+// Arguments of the kernels that stream a window or finish its chains.
+struct VerifyArgs {
+  const void* x;
+  const void* mq;
+  const void* mp;
+  const void* mq_bonus;
+  const float* sigma_bonus;
+  int64_t d;
+  int64_t chunk;
+  bool serial;           // a plain call: its stream waits for the work before it
+  int sms;               // the device's SMs (k_chain)
+  void* y;
+  uint64_t* tpart;       // [B, L, C] k_tiles' tagged partials (read through S.tpart)
+  ScanArgs S;
+};
+
 struct WsLayout {
   int vpt1;        // K1 16-byte vectors per thread per tensor
   int64_t chunk1;  // elements of a row per K1 tile
   int C1;          // K1 tiles per row
-  int64_t chunk4;  // K4 elements per tile
-  int C4;          // K4 tiles per chain
-  // tickets [B] u32 (fused kernel); two sets of tile partials [B, L, C1], 16 bytes
-  // each (the fused kernel's float2, in set 0, or k_tiles' tagged pair of words), each
-  // followed by its consumed tags [B, L, C1] u32; chain states; long-row partials
-  size_t ticket_off, part_off, part_set_bytes, cons_off, state_off, part4_off, total;
+  // two sets of k_tiles' partials [B, L, C1], 16 bytes each, each followed by its
+  // consumed tags [B, L, C1] u32
+  size_t part_off, part_set_bytes, cons_off, total;
 };
 
 WsLayout ws_layout(int B, int L, int64_t d, int dtype);
@@ -139,6 +133,9 @@ int verify_ex_impl(const void* x_draft, const void* mu_target, const void* mu_dr
 
 // Records a cudaError_t for sdv_last_cuda_error() (this host thread).
 void set_last_cuda_error(int err);
+
+// SMs of the current device (152 if it cannot be asked).
+int sm_count();
 
 // Largest number of mixture components of the analytic target.
 constexpr int kSdvMaxComponents = SDV_MAX_COMPONENTS;

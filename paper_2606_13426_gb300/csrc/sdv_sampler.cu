@@ -864,17 +864,6 @@ static GmmLaunch gmm_launch(int C, int64_t d, const void* means, bool rows_align
 
 static unsigned rows_grid(int n) { return (unsigned)std::max(1, (n + kGmmWarps - 1) / kGmmWarps); }
 
-static int sm_count() {
-  static int cache[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (cache[dev] == 0) {
-    int n = 0;
-    cache[dev] = (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) ? n : 152;
-  }
-  return cache[dev];
-}
-
 // Grid of k_round_target: one warp per RB row slots, at most four CTAs per SM (each
 // CTA stages the means once and strides over its share of the slots).
 static unsigned round_target_grid(const GmmLaunch& gl, int B, int L) {

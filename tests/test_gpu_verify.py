@@ -361,3 +361,113 @@ def test_device_special_functions(api):
     lam = np.exp(-0.5 * s64 * s64 - 0.5 * np.log(2 * np.pi) - log_ndtr(s64))
     gref = lam + s64
     assert np.all(np.abs(gp - gref) <= 1e-6 * np.maximum(1.0, np.abs(gref)) + 4e-7 * np.abs(s64))
+
+
+# ------------------------------------------------------------------ paths of a call
+def _path_case(api, kind, B, L, d, mode="block", seed=77, chains=None, shift=0, ragged=False, **kw):
+    """A call against the oracle; shift > 0 puts every window array that many elements off
+    its allocation's start (not 16-byte aligned: read element by element)."""
+    from gpu_helpers import to_dev
+    inp = W.make_verify_inputs(kind, B=B, L=L, d=d, per_chain_sigma=True)
+    m = OV.MODE_BLOCK if mode == "block" else OV.MODE_SAMPLE
+    okw = {}
+    if ragged:
+        rng = np.random.Generator(np.random.PCG64(B + d))
+        Leff = rng.integers(0, L + 1, B).astype(np.int32)
+        Leff[:2] = [0, L][:B]
+        okw["Leff"] = Leff
+        kw["L_eff"] = torch.from_numpy(Leff).cuda()
+    t = []
+    for name in ("x_draft", "mu_target", "mu_draft"):
+        v = to_dev(inp, name)
+        if shift:
+            buf = torch.zeros(v.numel() + shift, dtype=v.dtype, device="cuda")
+            buf[shift:] = v.reshape(-1)
+            v = buf[shift:].view(v.shape)
+        t.append(v)
+    r = api.verify(*t, torch.from_numpy(inp["sigma"]).cuda(), seed, mode, with_aux=True, **kw)
+    torch.cuda.synchronize()
+    ch = np.arange(B) if chains is None else np.asarray(chains)
+    g = {k: v.float().cpu().numpy()[ch] if v.dtype == torch.bfloat16 else v.cpu().numpy()[ch] for k, v in r.items()}
+    o = oracle_for(inp, seed, m, chains=ch, **okw)
+    compare(g, o, m, inp["dtype"])
+
+
+# Rows that start anywhere within a 16-byte vector: lengths around a vector, a tile (256 to
+# 1024 vectors, the last one straddled or not) and single elements; and arrays off their
+# 16-byte boundary.  The last row's last vector reaches past the array.
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("kind,d", [("pixel", 1), ("pixel", 3), ("pixel", 5), ("pixel", 1023), ("pixel", 1025),
+                                    ("pixel", 2047), ("pixel", 3073), ("pixel", 4097), ("pixel", 8189),
+                                    ("latent", 7), ("latent", 9), ("latent", 12), ("latent", 2047), ("latent", 2055),
+                                    ("latent", 4095), ("latent", 4097), ("latent", 6148)])
+def test_rows_off_vector_boundaries(api, kind, d, pipelined):
+    _path_case(api, kind, 3, 5, d, pipelined=pipelined)
+
+
+@pytest.mark.parametrize("kind,d,shift", [("pixel", 64, 1), ("pixel", 1027, 2), ("latent", 640, 3), ("latent", 4100, 4)])
+def test_arrays_off_vector_boundaries(api, kind, d, shift):
+    for pipelined in (False, True):
+        _path_case(api, kind, 4, 3, d, shift=shift, pipelined=pipelined)
+
+
+# One-kernel calls: 8, 4, 2 and 1 CTAs per chain (two per SM at most), one chain more than
+# that, fewer tiles than CTAs, finished chains and short windows, rows whose noise fits
+# a thread's registers or not.
+@pytest.mark.parametrize("kind,B,L,d", [("pixel", 1, 1, 16), ("pixel", 2, 7, 16384), ("latent", 38, 3, 4096),
+                                        ("latent", 39, 16, 1000), ("pixel", 77, 4, 3072), ("pixel", 153, 2, 4100),
+                                        ("pixel", 304, 3, 260), ("pixel", 305, 3, 260), ("tiny", 1, 64, 40),
+                                        ("pixel", 12, 33, 7000)])
+@pytest.mark.parametrize("mode", ["block", "sample"])
+def test_one_kernel_calls(api, kind, B, L, d, mode):
+    _path_case(api, kind, B, L, d, mode=mode, ragged=True)
+
+
+# Rows past one finishing CTA's: noise kept in shared memory and drawn twice, one CTA per
+# chain and several.
+@pytest.mark.parametrize("pipelined", [False, True])
+@pytest.mark.parametrize("kind,B,L,d,sample", [("pixel", 3, 8, 70001, None), ("latent", 9, 30, 60000, None),
+                                               ("pixel", 160, 2, 60000, [0, 1, 80, 159]),
+                                               ("pixel", 520, 1, 16400, [0, 5, 519])])
+def test_long_rows(api, kind, B, L, d, sample, pipelined):
+    _path_case(api, kind, B, L, d, chains=sample, pipelined=pipelined)
+
+
+def test_more_tile_sums_than_shared_memory_holds(api):
+    """64 steps of 203 tiles.  The ratios are those of the ratio kernel (the same sums in the
+    same order) and the acceptance that of the scan on them; rows of 830000 bf16 elements are
+    too long for the parity helper's 1e-5 on the ratios themselves (their terms add up to
+    1e5 and more, ell_error_bound)."""
+    from gpu_helpers import to_dev, y_tolerance
+    inp = W.make_verify_inputs("latent", B=1, L=64, d=830000)
+    t = [to_dev(inp, n) for n in ("x_draft", "mu_target", "mu_draft")] + [torch.from_numpy(inp["sigma"]).cuda()]
+    lr, dn = api.log_ratios(*t)
+    o = oracle_for(inp, 77, OV.MODE_BLOCK)
+    assert np.all(np.abs(lr.cpu().numpy() - o["ell"]) <= o["ell_bound"] + 4 * 2.0 ** -24 * np.abs(o["ell"]))
+    tau, _ = api.accept_scan(lr, dn, 77, "block")
+    for pipelined in (False, True):
+        r = api.verify(*t, 77, "block", pipelined=pipelined)
+        torch.cuda.synchronize()
+        assert torch.equal(r["log_ratio"], lr) and torch.equal(r["delta_norm"], dn)
+        assert torch.equal(r["accepted_len"], tau - 1)
+        assert r["accepted_len"].item() == o["accepted_len"][0]
+        assert np.all(np.abs(r["y"].float().cpu().numpy() - o["y"]) <= y_tolerance(o["y"], "bf16"))
+
+
+# Rows whose noise cache and static shared memory pass 48 KB together.
+@pytest.mark.parametrize("d", [11904, 12288, 12292])
+def test_rows_around_48_kb_of_shared_memory(api, d):
+    for pipelined in (False, True):
+        _path_case(api, "pixel", 2, 3, d, pipelined=pipelined)
+        _path_case(api, "pixel", 310, 1, d, chains=[0, 200, 309], pipelined=pipelined)
+
+
+def test_log_ratios_of_an_enormous_row(api):
+    """More tiles than one pass of a cluster holds (2048 of 4096 elements)."""
+    from gpu_helpers import to_dev
+    inp = W.make_verify_inputs("pixel", B=1, L=1, d=9_000_001)
+    lr, dn = api.log_ratios(to_dev(inp, "x_draft"), to_dev(inp, "mu_target"), to_dev(inp, "mu_draft"),
+                            torch.from_numpy(inp["sigma"]).cuda())
+    ell_o, dn_o = OV.log_ratios(inp["x_draft"], inp["mu_target"], inp["mu_draft"], inp["sigma"])
+    assert abs(lr.item() - ell_o.item()) <= 1e-5 * max(1.0, abs(ell_o.item()))
+    assert abs(dn.item() - dn_o.item()) <= 1e-5 * max(1.0, dn_o.item())
