@@ -334,12 +334,13 @@ size_t sdv_sampler_workspace_bytes(int B, int L, int64_t d);
  * `max_rounds` rounds have run.  One round: gamma_k = min(L, K - k) draft steps, the
  * parallel target call at yhat_k .. yhat_{k+gamma_k}, sdv_verify_ex (residual or bonus
  * step), then k <- min(k + tau, K); a window that reaches K takes no bonus step.
- * The rounds run as one CUDA graph launched on `stream`: a while node whose body is
- * one round (draft, target call, verification, update), the round counter and seed
- * held in the workspace and the loop ended on the device once no chain is active or
- * max_rounds rounds ran.  Unlike the other entry points this call synchronises (it
- * waits for the graph to read back the number of rounds), so it cannot itself be
- * captured into a graph.
+ * Rows of up to 4096 elements whose chains are resident at once (a thread block each): one
+ * kernel runs all rounds.  Else the rounds run as one CUDA graph launched on `stream`, a
+ * while node whose body is one round (draft, target call, verification, update), the round
+ * counter and seed held in the workspace and the loop ended on the device once no chain is
+ * active or max_rounds rounds ran; a few rounds in which no chain can finish are launched
+ * one after another.  Unlike the other entry points this call synchronises (it waits to
+ * read back the number of rounds), so it cannot itself be captured into a graph.
  *   y_out [B, d] fp32 out: the chains' states (Y_K when finished)
  *   k_out [B], chain_rounds_out [B], tau_sum_out [B] int32 out or NULL: step reached,
  *     rounds taken part in, sum of tau over those rounds
@@ -356,8 +357,8 @@ int sdv_sampler_run(int B, int L, int64_t d, const float *means, const float *lo
  * Host-driven rounds: the same sampler as sdv_sampler_run, one call per round.
  * sdv_sampler_begin draws Y_0 and makes the initial target call (the chains'
  * bookkeeping and round state live in the workspace); each sdv_sampler_round
- * enqueues one round (the same kernels, in the same order, as one iteration of
- * sdv_sampler_run's graph, so that begin + R rounds + end gives the same results
+ * enqueues one round (the kernel, or the kernels in their order, of one round of
+ * sdv_sampler_run, so that begin + R rounds + end gives the same results
  * as sdv_sampler_run with max_rounds = R while a chain is active; a round with no
  * active chain only advances the round counter); sdv_sampler_end synchronises
  * `stream` and returns the same outputs as sdv_sampler_run.  Every round must pass

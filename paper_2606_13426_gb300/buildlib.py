@@ -18,7 +18,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIBDIR = os.path.join(PKG, "lib")
 LIBNAME = "libspecdiff.so"
-SOURCES = ["sdv_verify.cu", "sdv_chain_f32.cu", "sdv_chain_bf16.cu", "sdv_sampler.cu", "sdv_noalloc.cu"]
+SOURCES = ["sdv_verify.cu", "sdv_chain_f32.cu", "sdv_chain_bf16.cu", "sdv_sampler.cu", "sdv_rounds_c8.cu",
+           "sdv_rounds_c16.cu", "sdv_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I" + INCLUDE,
               "-I" + CSRC]

@@ -233,6 +233,18 @@ def test_first_rounds_other_shapes(api, d, C):
     _first_rounds(api, OV.MODE_BLOCK, "free", d, C, Bn=96)
 
 
+# Edges of the round kernel: row lengths around its thread counts and groups per thread, odd
+# tails, windows longer than the noise drawn ahead, one row per pass (more chains than are
+# resident at once) or several, and the longest rows it takes and the next (round graph).
+@pytest.mark.parametrize("Bn,d,C,L", [(2, 3, 1, 4), (9, 128, 8, 5), (9, 129, 9, 5), (40, 256, 16, 4), (40, 257, 2, 33),
+                                      (33, 513, 8, 64), (460, 600, 8, 4), (460, 516, 12, 4), (1830, 200, 8, 4),
+                                      (12, 1026, 8, 6), (12, 2048, 9, 12), (12, 2052, 8, 4), (6, 4096, 8, 4),
+                                      (6, 4093, 3, 4), (6, 4100, 8, 4), (6, 4099, 12, 4)])
+@pytest.mark.parametrize("mode,drafter", [(OV.MODE_BLOCK, "frozen"), (OV.MODE_SAMPLE, "free")])
+def test_round_kernel_edges(api, Bn, d, C, L, mode, drafter):
+    _first_rounds(api, mode, drafter, d, C, Bn=Bn, L=L, K=200, chains=np.unique(np.linspace(0, Bn - 1, 12).astype(int)))
+
+
 def _check_law(y, m, var, n_sigma=4.0):
     n = y.shape[0]
     assert np.all(np.abs(y.mean(0) - m) < n_sigma * math.sqrt(var / n))
