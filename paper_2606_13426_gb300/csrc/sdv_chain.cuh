@@ -222,6 +222,10 @@ __device__ __forceinline__ void finish_cluster(const VerifyArgs& A, int b, int c
   bool have_P = false;
   // ---- acceptance (the first CTA)
   if (rank == 0 && warp < scanners) {
+    // the coins, which warp 0 has drawn (k_finish_long comes here without a barrier since;
+    // warps that decide differently would part for ever)
+    if (scanners > 1) asm volatile("bar.sync 2, %0;" ::"r"(32 * scanners) : "memory");
+    else __syncwarp();
     R = scan_load(A.S, b, false, tile_s);
     const float leta[2] = {fs.leta[lane], fs.leta[lane + 32]};
     const ScanOut so = scan_decide(A.S, b, R, leta, co);

@@ -424,9 +424,11 @@ def test_one_kernel_calls(api, kind, B, L, d, mode):
 
 
 # Rows past one finishing CTA's: noise kept in shared memory and drawn twice, one CTA per
-# chain and several.
+# chain and several; and the shortest of them, whose noise is drawn as fast as the coins that
+# every scanning warp waits for.
 @pytest.mark.parametrize("pipelined", [False, True])
 @pytest.mark.parametrize("kind,B,L,d,sample", [("pixel", 3, 8, 70001, None), ("latent", 9, 30, 60000, None),
+                                               ("pixel", 20, 19, 16388, [0, 7, 13, 19]),
                                                ("pixel", 160, 2, 60000, [0, 1, 80, 159]),
                                                ("pixel", 520, 1, 16400, [0, 5, 519])])
 def test_long_rows(api, kind, B, L, d, sample, pipelined):
