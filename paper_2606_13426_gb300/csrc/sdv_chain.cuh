@@ -412,9 +412,9 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
 // adds them in tile order (as scan_load does, so that the ratios equal a whole call's) and
 // writes ell_j and |Delta_j|.
 template <typename T, int ROWS, int VPT>
-__global__ void __launch_bounds__(kK1Threads, 3) k_ratios(VerifyArgs A, int cl, int span) {
+__global__ void __launch_bounds__(kK1Threads, VPT == 1 ? 6 : 3) k_ratios(VerifyArgs A, int cl, int span) {
   constexpr int NW = kK1Threads / 32;
-  constexpr int NB = tiles_in_flight(VPT);
+  constexpr int NB = VPT == 1 ? 1 : tiles_in_flight(VPT);   // rows of one such tile are a tile each
   extern __shared__ float4 dyn_s[];
   const int L = A.S.L, C = A.S.C;
   const int64_t row = blockIdx.x / cl;
@@ -509,6 +509,9 @@ static int max_clusters(int cl, int per_sm) {
 // a CTA, 24.5 us here and 25.2 split; 200 x 8 x 4096, 384 KB, 27.7 and 26.3; 100 x 8 x 10000,
 // 313 KB, 34.6 and 29.0; 56 x 17 x 63432, 2.5 MB, 164 and 138.
 constexpr int64_t kChainBytes = 300 * 1024;
+// And at most 16 groups of four of the row for a thread: longer rows, of short windows, are
+// finished by more threads (88 x 1 x 96920 fp32 112 us here, 62 by k_finish_long).
+constexpr int64_t kChainGroups = 16 * (kK1Threads - 32);
 static int chain_cluster(int B, int L, int C, int64_t d, int es) {
   const int sms = sm_count();
   if (B > kChainPerSm * sms) return 0;
@@ -584,7 +587,7 @@ cudaError_t launch_chain(const VerifyArgs& A, int B, int L, int vpt, int rows, b
   const size_t most = ((size_t)L * C + cl - 1) / cl;
   const int64_t ng = (A.d + 3) / 4, per = (ng + cl - 1) / cl;
   const size_t smem = 16 * ((most * (kK1Threads / 32) + (size_t)L * C + 1) / 2) + sizeof(float4) * (size_t)per;
-  if (smem > kChainSmemMax) return cudaSuccess;
+  if (smem > kChainSmemMax || per > kChainGroups) return cudaSuccess;
   *taken = true;
   return per <= (int64_t)kOwn * (kK1Threads - 32) ? launch_t<T, kHoldAll>(A, B, cl, vpt, rows, smem, s)
                                                   : launch_t<T, kHoldNoise>(A, B, cl, vpt, rows, smem, s);
@@ -595,25 +598,31 @@ static cudaError_t launch_long_t(const VerifyArgs& A, int B, int cl, size_t tile
   const int stage = tiles <= kFinishSmemMax / 2;
   if (!stage) tiles = 0;
   // many CTAs: two per SM, as far as the noise allows
-  if (tiles + noise <= (NT == kLongThreads ? kFinishSmemMax : kChainSmemMax))
+  if (A.S.residual_kind != SDV_RESIDUAL_REFLECTION &&   // which draws noise only where delta = 0
+      tiles + noise <= (NT == kLongThreads ? kFinishSmemMax : kChainSmemMax))
     return launch_cluster(k_finish_long<T, VEC4, kHoldNoise, NT>, A, B, cl, tiles + noise, s, NT, stage);
   return launch_cluster(k_finish_long<T, VEC4, kHoldNothing, NT>, A, B, cl, tiles, s, NT, stage);
 }
 
 template <typename T>
 cudaError_t launch_finish_long(const VerifyArgs& A, int B, int L, bool vec4, cudaStream_t s) {
-  // few chains: as many CTAs per chain as leave every cluster a place at once, one CTA per SM;
-  // many: four, so that the last wave of them is short
-  const bool few = B <= sm_count();
-  int cl = few ? 6 : 4;
-  while (few && cl > 1 && B > max_clusters(cl, 1)) --cl;
-  const size_t tiles = 16 * (((size_t)L * A.S.C + 1) / 2);
-  const size_t noise = sizeof(float4) * (size_t)(((A.d + 3) / 4 + cl - 1) / cl);
-  if (few)
-    return vec4 ? launch_long_t<T, true, kLongThreads>(A, B, cl, tiles, noise, s)
-                : launch_long_t<T, false, kLongThreads>(A, B, cl, tiles, noise, s);
-  return vec4 ? launch_long_t<T, true, kLongThreadsMany>(A, B, cl, tiles, noise, s)
-              : launch_long_t<T, false, kLongThreadsMany>(A, B, cl, tiles, noise, s);
+  // Few chains: as many CTAs per chain, of 512 threads, as leave every cluster a place at once,
+  // one CTA per SM.  Where that leaves a chain one CTA, or too little shared memory for its
+  // noise, four CTAs of 256 threads, two to an SM, so that the last wave of them is short; or
+  // eight, where only those hold the noise.  (88 chains of one step of 96919 bf16 elements: 66 us
+  // with eight, 68 with four, 124 with one of 512 threads; 150 x 1 x 50000 fp32 56 with four, 69
+  // with one; but 56 x 17 x 63432 140 with two of 512 threads, 168 with four of 256.)
+  size_t tiles = 16 * (((size_t)L * A.S.C + 1) / 2);
+  const auto noise = [&](int c) { return sizeof(float4) * (size_t)(((A.d + 3) / 4 + c - 1) / c); };
+  const auto fits = [&](int c, size_t most) { return (tiles <= kFinishSmemMax / 2 ? tiles : 0) + noise(c) <= most; };
+  int cl = B <= 8 ? 8 : 6;
+  while (cl > 1 && B > max_clusters(cl, 1)) --cl;
+  if (cl > 1 && (fits(cl, kFinishSmemMax) || !fits(8, kChainSmemMax)))
+    return vec4 ? launch_long_t<T, true, kLongThreads>(A, B, cl, tiles, noise(cl), s)
+                : launch_long_t<T, false, kLongThreads>(A, B, cl, tiles, noise(cl), s);
+  cl = fits(4, kChainSmemMax) || !fits(8, kChainSmemMax) ? 4 : 8;
+  return vec4 ? launch_long_t<T, true, kLongThreadsMany>(A, B, cl, tiles, noise(cl), s)
+              : launch_long_t<T, false, kLongThreadsMany>(A, B, cl, tiles, noise(cl), s);
 }
 
 template <typename T>

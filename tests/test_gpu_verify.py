@@ -430,6 +430,8 @@ def test_one_kernel_calls(api, kind, B, L, d, mode):
 @pytest.mark.parametrize("kind,B,L,d,sample", [("pixel", 3, 8, 70001, None), ("latent", 9, 30, 60000, None),
                                                ("pixel", 20, 19, 16388, [0, 7, 13, 19]),
                                                ("pixel", 160, 2, 60000, [0, 1, 80, 159]),
+                                               ("latent", 88, 1, 60003, [0, 40, 87]),
+                                               ("pixel", 40, 1, 120001, [0, 39]),
                                                ("pixel", 520, 1, 16400, [0, 5, 519])])
 def test_long_rows(api, kind, B, L, d, sample, pipelined):
     _path_case(api, kind, B, L, d, chains=sample, pipelined=pipelined)
