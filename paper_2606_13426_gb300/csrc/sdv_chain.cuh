@@ -410,7 +410,10 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
 // ---------------------------------------------------------------- log ratios alone
 // One cluster of CTAs per row (chain b, step j): its tiles' sums meet in the first CTA, which
 // adds them in tile order (as scan_load does, so that the ratios equal a whole call's) and
-// writes ell_j and |Delta_j|.
+// writes ell_j and |Delta_j|.  Bound by HBM for long rows (64 chains x 16 steps x 16384 bf16
+// elements, 100.7 MB: 26.7 us with ticket counters and their memset, 18.5 now), by the CTAs'
+// latency for many short ones, hence six per SM where a row is one small tile (471 x 18 rows
+// of 576 bf16 elements: 51 us with three per SM, 24.5 with six).
 template <typename T, int ROWS, int VPT>
 __global__ void __launch_bounds__(kK1Threads, VPT == 1 ? 6 : 3) k_ratios(VerifyArgs A, int cl, int span) {
   constexpr int NW = kK1Threads / 32;
