@@ -566,7 +566,7 @@ static cudaError_t launch_t(const VerifyArgs& A, int B, int cl, int vpt, int row
   // tiles have at most two vectors)
   constexpr bool kSmall = HOLD == kHoldAll;
   if constexpr (kSmall) {
-    if (vpt == 1) { SDV_VPT(1); }
+    if (vpt == 1) return launch_cluster(k_chain<T, kRowsAligned, 1, true, HOLD>, A, B, cl, smem, s, kK1Threads);
   }
   if constexpr (kSmall || sizeof(T) == 2) {
     if (vpt == 2) { SDV_VPT(2); }
@@ -587,6 +587,10 @@ cudaError_t launch_chain(const VerifyArgs& A, int B, int L, int vpt, int rows, b
   const int C = A.S.C;
   const int cl = chain_cluster(B, L, C, A.d, (int)sizeof(T));
   if (cl == 0 || (rows == kRowsAligned && !vec4)) return cudaSuccess;
+  // one-vector tiles of rows off vector boundaries stream better spread over all SMs: 160 chains x
+  // 25 steps x 1501 bf16 elements 38.0 us here, 23.4 by k_tiles, 4 x 16 x 1501 12.8 and 12.5
+  // (but 300 x 12 x 901 fp32 19.3 and 20.6)
+  if (rows == kRowsUnaligned && vpt == 1) return cudaSuccess;
   const size_t most = ((size_t)L * C + cl - 1) / cl;
   const int64_t ng = (A.d + 3) / 4, per = (ng + cl - 1) / cl;
   const size_t smem = 16 * ((most * (kK1Threads / 32) + (size_t)L * C + 1) / 2) + sizeof(float4) * (size_t)per;
