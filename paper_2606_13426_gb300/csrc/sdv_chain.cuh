@@ -515,6 +515,7 @@ constexpr int64_t kChainBytes = 300 * 1024;
 // And at most 16 groups of four of the row for a thread: longer rows, of short windows, are
 // finished by more threads (88 x 1 x 96920 fp32 112 us here, 62 by k_finish_long).
 constexpr int64_t kChainGroups = 16 * (kK1Threads - 32);
+constexpr size_t kChainTiles = 16;   // tiles of a CTA, of rows read as vectors
 static int chain_cluster(int B, int L, int C, int64_t d, int es) {
   const int sms = sm_count();
   if (B > kChainPerSm * sms) return 0;
@@ -592,6 +593,10 @@ cudaError_t launch_chain(const VerifyArgs& A, int B, int L, int vpt, int rows, b
   // (but 300 x 12 x 901 fp32 19.3 and 20.6)
   if (rows == kRowsUnaligned && vpt == 1) return cudaSuccess;
   const size_t most = ((size_t)L * C + cl - 1) / cl;
+  // nor many tiles of whole vectors one batch after another: 160 x 25 x 1024 bf16 elements 27.1 us
+  // here, 21.0 by k_tiles, 160 x 25 x 512 fp32 22.9 and 19.9; twelve tiles, 300 x 12 x 1024 fp32,
+  // 19.2 and 21.0; read by element, 160 x 25 x 256 fp32, 17.1 and 20.1
+  if (rows == kRowsAligned && most > kChainTiles) return cudaSuccess;
   const int64_t ng = (A.d + 3) / 4, per = (ng + cl - 1) / cl;
   const size_t smem = 16 * ((most * (kK1Threads / 32) + (size_t)L * C + 1) / 2) + sizeof(float4) * (size_t)per;
   if (smem > kChainSmemMax || per > kChainGroups) return cudaSuccess;
