@@ -65,7 +65,7 @@ struct ScanArgs {
   const uint64_t* tpart;  // k_tiles: [B, L, C] pairs of words (S1 | tag << 32, S2 | tag << 32)
   uint32_t* consumed;     // [B, L, C] beside tpart: the tag of the partial last read from each slot
   uint32_t tag;           // this call's tag of its k_tiles partials (never 0)
-  bool fresh_set;         // the set held another layout before: k_tiles waits before its stores
+  bool fresh_set;         // the first call on the set since another layout (PartialSets): k_tiles waits before its stores
   int C;
   const float* sigma;
   int64_t sstride;

@@ -19,7 +19,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <mutex>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -28,6 +27,7 @@
 #include "sdv_device.cuh"
 #include "sdv_host.h"
 #include "sdv_scan.cuh"
+#include "sdv_sets.h"
 #include "sdv_tiles.cuh"
 #include "sdv_finish.cuh"
 #include "sdv_chain.h"
@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(kK1Threads, tile_min_blocks(VPT)) k_tiles(Veri
     const float2 t = block_sum2<kK1Threads>(sm.x, sm.y, red);
     if (threadIdx.x == 0) {
       // the slot's partial has not been read yet by the call that wrote it (which may
-      // still be finishing, since calls overlap), or this set held another layout:
-      // wait for the previous kernel, whose completion implies every earlier call's
+      // still be finishing, since calls overlap), or a call of another layout may have
+      // written here: wait for the previous kernel, whose completion implies every earlier call's
       // (in practice the slot was read long ago)
       if (A.S.fresh_set || held != taken) griddep_wait();
       // S1 and S2 each share an 8-byte word with the call's tag; each word is written
@@ -461,31 +461,7 @@ static uint32_t next_partial_tag() {
   return t;
 }
 
-// The set of partials a call on `workspace` uses: the other one than the previous call
-// on that workspace (remembered for the last kPartialSetSlots workspaces; a forgotten
-// workspace starts again at set 0, which at worst makes a stream CTA wait for the
-// previous kernel before its store).
-// `fresh` when the set's last user on this workspace had another layout (or is
-// unknown): the stream then waits for the previous kernel before it stores.
-constexpr int kPartialSetSlots = 64;
-static int next_partial_set(const void* workspace, uint64_t layout, bool* fresh) {
-  struct Entry {
-    const void* ws;
-    int next;
-    uint64_t layout[2];
-  };
-  static std::mutex mu;
-  static Entry tab[kPartialSetSlots] = {};
-  const size_t h = (reinterpret_cast<uintptr_t>(workspace) >> 8) % kPartialSetSlots;
-  std::lock_guard<std::mutex> lock(mu);
-  Entry& e = tab[h];
-  if (e.ws != workspace) e = Entry{workspace, 0, {0u, 0u}};
-  const int set = e.next;
-  *fresh = e.layout[set] != layout;
-  e.layout[set] = layout;
-  e.next ^= 1;
-  return set;
-}
+static PartialSets g_partial_sets;
 
 // Enqueue the whole step (or, with ratios_only, the log-ratio pass) for validated args.
 static int enqueue_verify(const void* x_draft, const void* mu_target, const void* mu_draft,
@@ -561,10 +537,9 @@ static int enqueue_verify(const void* x_draft, const void* mu_target, const void
   const bool long_rows = ng > kPipeMaxGroups;
   // k_tiles + k_finish: tagged partials in the set after the one this workspace's
   // previous call used, no counters
-  // the layout key: the slot count and the set's size (never 0)
-  const uint64_t layout = ((uint64_t)B * L * w.C1 << 24) ^ (uint64_t)w.part_set_bytes ^ 1u;
+  const uint64_t layout = (uint64_t)B * L * w.C1;   // the slots of a set, which fix both sets' places
   bool fresh = true;
-  char* set = ws + w.part_off + (size_t)next_partial_set(workspace, layout, &fresh) * w.part_set_bytes;
+  char* set = ws + w.part_off + (size_t)g_partial_sets.next(workspace, layout, &fresh) * w.part_set_bytes;
   S.fresh_set = fresh;
   A.tpart = (uint64_t*)set;
   S.tpart = A.tpart;

@@ -195,3 +195,16 @@ def test_pipelined_calls_reuse_a_workspace_across_sizes(api):
     for i, sh in enumerate(order):
         fresh = torch.zeros(api.workspace_bytes(*sh, torch.float32), dtype=torch.uint8, device="cuda")
         _same(piped[i], _call(api, sets[sh], 900 + i, "block", fresh))
+
+
+def test_pipelined_large_and_small_calls_in_turn(api):
+    """A small call's second set of partials lies inside a large call's first: every call
+    after a change of sizes waits for the call before it (against plain calls)."""
+    large, small = (64, 8, 3072), (25, 8, 3072)
+    sets = {sh: _sets("pixel", 1, *sh, False)[0] for sh in (large, small)}
+    ws = torch.zeros(api.workspace_bytes(*large, torch.float32), dtype=torch.uint8, device="cuda")
+    order = [large, small, large] * 6
+    piped = [_call(api, sets[sh], 1100 + i, "block", ws, pipelined=True) for i, sh in enumerate(order)]
+    torch.cuda.synchronize()
+    for i, sh in enumerate(order):
+        _same(piped[i], _call(api, sets[sh], 1100 + i, "block", ws))
