@@ -349,17 +349,10 @@ __global__ void __launch_bounds__(kK1Threads, kChainPerSm) k_chain(VerifyArgs A,
 // Threads of k_finish_long: 512 where every CTA has an SM to itself, else 256.
 constexpr int kLongThreads = 512, kLongThreadsMany = 256;
 
-// The slots of chain b's partials are free for the next call that writes this set.
-__device__ __forceinline__ void release_slots(const VerifyArgs& A, int b, int g) {
-  const int64_t s0 = (int64_t)b * A.S.L * A.S.C;
-  for (int t = threadIdx.x; t < g * A.S.C; t += blockDim.x)
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.S.consumed + s0 + t), "r"(A.S.tag) : "memory");
-}
-
 // The end of a call whose window k_tiles streams, for rows too long for one finishing CTA
 // (k_finish): a cluster per chain.  Its first CTA reads the chain's partials with all its
-// threads (the tags tell this call's; a stale one makes it wait for k_tiles) and releases
-// their slots; the rest is k_chain's.  (stage = 0: sums of more tiles than shared memory
+// threads (the tags tell this call's; a stale one, or a fresh set, makes it wait for k_tiles)
+// and frees their slots; the rest is k_chain's.  (stage = 0: sums of more tiles than shared memory
 // holds are read by its first warp.)
 template <typename T, bool VEC4, int HOLD, int NT>
 __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int stage) {
@@ -378,16 +371,15 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
   float2* tile_s = stage ? reinterpret_cast<float2*>(dyn_s) : nullptr;   // [L C]
   float4* g_s = dyn_s + (stage ? (L * C + 1) / 2 : 0);
   const RowSlice sl = cluster_slice(A.d, cl, rank);
-  if (rank == 0 && !stage) griddep_wait();                // warp 0 reads the partials itself
+  uint64_t* const p = A.S.tpart + 2 * ((int64_t)b * L * C);
+  if (rank == 0 && (!stage || A.S.fresh_set)) griddep_wait();   // !stage: warp 0 reads the partials itself
   if (rank == 0 && stage) {
-    const int64_t s0 = (int64_t)b * L * C;
-    const ulonglong2* p = reinterpret_cast<const ulonglong2*>(A.tpart) + s0;
     auto fetch = [&](bool check) {
       int stale = 0;
 #pragma unroll 4
       for (int t = threadIdx.x; t < g * C; t += NT) {
-        const ulonglong2 v = __ldcg(p + t);
-        if (check && ((uint32_t)(v.x >> 32) != A.S.tag || (uint32_t)(v.y >> 32) != A.S.tag)) stale = 1;
+        const ulonglong2 v = slot_read(p + 2 * t);
+        if (check && !slot_holds(v, A.S.tag)) stale = 1;
         tile_s[t] = make_float2(__uint_as_float((uint32_t)v.x), __uint_as_float((uint32_t)v.y));
       }
       return __syncthreads_or(stale);
@@ -396,14 +388,14 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
       griddep_wait();
       (void)fetch(false);
     }
-    release_slots(A, b, g);
+    slots_free(p, threadIdx.x, NT, g * C);
   }
   if (cl > 1) cluster_wait();
   finish_ahead<HOLD>(A, b, rank, sl, g_s, fs);
   finish_cluster<T, VEC4, HOLD, NT>(A, b, cl, rank, tile_s, sl, g_s, fs);
   if (rank == 0 && !stage) {
     __syncthreads();
-    release_slots(A, b, g);
+    slots_free(p, threadIdx.x, NT, g * C);
   }
 }
 

@@ -62,10 +62,9 @@ struct ChainState {
 };
 
 struct ScanArgs {
-  const uint64_t* tpart;  // k_tiles: [B, L, C] pairs of words (S1 | tag << 32, S2 | tag << 32)
-  uint32_t* consumed;     // [B, L, C] beside tpart: the tag of the partial last read from each slot
-  uint32_t tag;           // this call's tag of its k_tiles partials (never 0)
-  bool fresh_set;         // the first call on the set since another layout (PartialSets): k_tiles waits before its stores
+  uint64_t* tpart;        // k_tiles' slots, [B, L, C] pairs of words (S1 | tag << 32, S2 | tag << 32)
+  uint32_t tag;           // this call's tag of its k_tiles partials (never 0: a free slot's tag)
+  bool fresh_set;         // the first call on the set since another layout (PartialSets): its contents are unknown
   int C;
   const float* sigma;
   int64_t sstride;
@@ -102,7 +101,6 @@ struct VerifyArgs {
   bool serial;           // a plain call: its stream waits for the work before it
   int sms;               // the device's SMs (k_chain)
   void* y;
-  uint64_t* tpart;       // [B, L, C] k_tiles' tagged partials (read through S.tpart)
   ScanArgs S;
 };
 
@@ -110,9 +108,8 @@ struct WsLayout {
   int vpt1;        // K1 16-byte vectors per thread per tensor
   int64_t chunk1;  // elements of a row per K1 tile
   int C1;          // K1 tiles per row
-  // two sets of k_tiles' partials [B, L, C1], 16 bytes each, each followed by its
-  // consumed tags [B, L, C1] u32
-  size_t part_off, part_set_bytes, cons_off, total;
+  // two sets of k_tiles' slots [B, L, C1], 16 bytes each
+  size_t part_off, part_set_bytes, total;
 };
 
 WsLayout ws_layout(int B, int L, int64_t d, int dtype);

@@ -42,6 +42,39 @@ __device__ __forceinline__ UParams shfl_params(const UParams& P, int src) {
   return R;
 }
 
+// The slot of a tile's partial: S1 and S2, each in an 8-byte word below the tag of the call
+// that stored it (words are read and written whole, so that a tag vouches for the sum beside
+// it).  Its reader frees the slot by clearing both words, the second with release: a replayed
+// call, whose tag is the one it was captured with, then finds no partial of an earlier replay
+// there, and whoever sees the second word clear (acquire) may store.
+__device__ __forceinline__ ulonglong2 slot_read(const uint64_t* p) {
+  ulonglong2 v;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ bool slot_holds(const ulonglong2& v, uint32_t tag) {
+  return (uint32_t)(v.x >> 32) == tag && (uint32_t)(v.y >> 32) == tag;
+}
+// (One word: asking for both by one 16-byte acquire made eight pipelined latent calls take
+// 185.7 us, by two acquires 193; this way 172.6.)
+__device__ __forceinline__ bool slot_is_free(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p + 1) : "memory");
+  return (uint32_t)(v >> 32) == 0u;
+}
+__device__ __forceinline__ void slot_store(uint64_t* p, uint32_t tag, float2 s) {
+  const unsigned long long t = (unsigned long long)tag << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(t | __float_as_uint(s.x)),
+               "l"(t | __float_as_uint(s.y)) : "memory");
+}
+// Frees slots t0, t0 + dt, ... below n, once a barrier has shown that they are read.
+__device__ __forceinline__ void slots_free(uint64_t* p, int t0, int dt, int n) {
+  for (int t = t0; t < n; t += dt) {
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t), "l"(0ull) : "memory");
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t + 1), "l"(0ull) : "memory");
+  }
+}
+
 // Per-lane values of one chain's window, held by one warp: step j in lane j & 31 of
 // segment j >> 5 (L <= 64).
 struct ScanRegs {
@@ -63,9 +96,8 @@ __device__ __forceinline__ bool scan_step(ScanRegs& R, int q, float a1, float a2
 
 // Loads chain b's ell_j and |Delta_j|: from the tile partials (S1, S2 of every tile of
 // the row, read through L2; or `tiles`, the chain's [L, C] in shared memory) and sigma,
-// or from given arrays.  k_tiles partials carry the
-// call's tag in each 8-byte word (written whole); with check_tags, R.stale reports a
-// word whose tag is not this call's.  Called by a full warp; reads only.
+// or from given arrays.  With check_tags, R.stale reports a slot that does not hold this
+// call's partial.  Called by a full warp; reads only.
 __device__ __forceinline__ ScanRegs scan_load(const ScanArgs& A, int b, bool check_tags = true,
                                               const float2* tiles = nullptr) {
   const unsigned FULL = 0xffffffffu;
@@ -91,14 +123,19 @@ __device__ __forceinline__ ScanRegs scan_load(const ScanArgs& A, int b, bool che
             a2 += tiles[j * A.C + c].y;
           }
         } else {
-          const int64_t s0 = ((int64_t)b * L + j) * A.C;
-          const ulonglong2* p = reinterpret_cast<const ulonglong2*>(A.tpart) + s0;
-#pragma unroll 4
-          for (int c = 0; c < A.C; ++c) {
-            const ulonglong2 t = __ldcg(p + c);
-            if (check_tags && ((uint32_t)(t.x >> 32) != A.tag || (uint32_t)(t.y >> 32) != A.tag)) stale = true;
-            a1 += __uint_as_float((uint32_t)t.x);
-            a2 += __uint_as_float((uint32_t)t.y);
+          const uint64_t* p = A.tpart + 2 * (((int64_t)b * L + j) * A.C);
+          for (int c0 = 0; c0 < A.C; c0 += 4) {   // four loads in flight
+            ulonglong2 t[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) t[u] = slot_read(p + 2 * min(c0 + u, A.C - 1));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+              if (c0 + u < A.C) {
+                if (check_tags && !slot_holds(t[u], A.tag)) stale = true;
+                a1 += __uint_as_float((uint32_t)t[u].x);
+                a2 += __uint_as_float((uint32_t)t[u].y);
+              }
+            }
           }
         }
         bad |= scan_step(R, q, a1, a2, A.sigma[(int64_t)b * A.sstride + j]);

@@ -35,14 +35,6 @@
 namespace sdv {
 
 // ---------------------------------------------------------------- stream and finish
-// The tag of the partial in slot `tile` of this call's set and the tag its reader
-// released after reading it (acquire: the reader's loads of the slot happen before
-// anything this thread does next).
-__device__ __forceinline__ void slot_state(const VerifyArgs& A, int64_t tile, uint32_t& held, uint32_t& taken) {
-  held = __ldcg(reinterpret_cast<const unsigned int*>(A.tpart + 2 * tile) + 1);
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(taken) : "l"(A.S.consumed + tile) : "memory");
-}
-
 // The stream: one tile per CTA; its (S1, S2) is stored with the call's tag.  Bound by HBM
 // (8 rows of 3072 floats for 256 chains, 75.5 MB, in about 11 us alone, 6.9 TB/s).  (Two or
 // four software-pipelined tiles per CTA measured slower: 17.4 / 20.1 us against 16.5 us per
@@ -64,39 +56,34 @@ __global__ void __launch_bounds__(kK1Threads, tile_min_blocks(VPT)) k_tiles(Veri
   if (j < g) {  // CTA-uniform
     const int64_t e0 = (int64_t)c * A.chunk;
     const int64_t e1 = min(e0 + A.chunk, A.d);
-    // the tag now in this CTA's slot and the tag last consumed from it, loaded by thread
-    // 0 once its tile loads are in flight (the acquire orders only what follows it) and
-    // compared before the store
-    uint32_t held = 0u, taken = 0u;
+    // whether this CTA's slot is free, asked by thread 0 once its tile loads are in flight
+    // (the acquire orders only what follows it)
+    uint64_t* const slot = A.S.tpart + 2 * tile;
+    bool is_free = false;
     float2 sm;
     if (ROWS == kRowsAligned) {
       TileBuf<VPT> B;
       tile_issue<T, VPT>((const T*)A.x, (const T*)A.mq, (const T*)A.mp, r * A.d, e0, e1, B);
-      if (threadIdx.x == 0) slot_state(A, tile, held, taken);
+      if (threadIdx.x == 0) is_free = slot_is_free(slot);
       sm = tile_fma<T, VPT>(B);
     } else if (ROWS == kRowsUnaligned) {
       TileBuf<VPT> B;
       EdgeBuf E;
       unaligned_issue<T, VPT>((const T*)A.x, (const T*)A.mq, (const T*)A.mp, r * A.d, A.d, c, C, B, E);
-      if (threadIdx.x == 0) slot_state(A, tile, held, taken);
+      if (threadIdx.x == 0) is_free = slot_is_free(slot);
       sm = unaligned_fma<T, VPT>(B, E);
     } else {
-      if (threadIdx.x == 0) slot_state(A, tile, held, taken);
+      if (threadIdx.x == 0) is_free = slot_is_free(slot);
       sm = tile_sums<T>((const T*)A.x, (const T*)A.mq, (const T*)A.mp, r * A.d, e0, e1);
     }
     const float2 t = block_sum2<kK1Threads>(sm.x, sm.y, red);
     if (threadIdx.x == 0) {
       // the slot's partial has not been read yet by the call that wrote it (which may
       // still be finishing, since calls overlap), or a call of another layout may have
-      // written here: wait for the previous kernel, whose completion implies every earlier call's
-      // (in practice the slot was read long ago)
-      if (A.S.fresh_set || held != taken) griddep_wait();
-      // S1 and S2 each share an 8-byte word with the call's tag; each word is written
-      // whole (a vector of two 8-byte elements), so k_finish can tell this call's
-      // partials from those a previous call left in the slot
-      const unsigned long long tg = (unsigned long long)A.S.tag << 32;
-      reinterpret_cast<ulonglong2*>(A.tpart)[tile] =
-          make_ulonglong2(tg | __float_as_uint(t.x), tg | __float_as_uint(t.y));
+      // written here: wait for the previous kernel, whose completion implies every
+      // earlier call's (in practice the slot was read long ago)
+      if (A.S.fresh_set || !is_free) griddep_wait();
+      slot_store(slot, A.S.tag, t);
     }
   }
   if (blockIdx.x == 0) {
@@ -114,8 +101,8 @@ __global__ void __launch_bounds__(kK1Threads, tile_min_blocks(VPT)) k_tiles(Veri
 // only after every k_tiles CTA has stored its partial and exited or triggered; the tags
 // confirm that each one read is this call's, else the warp waits for k_tiles to
 // complete and reads them again) and scans the chain, while the other warps draw the
-// residual's G into shared memory (dynamic, (d + 3)/4 float4) and warp 1 releases the
-// chain's slots to the next call that writes this set; then warp 0 draws U while the
+// residual's G into shared memory (dynamic, (d + 3)/4 float4) and warp 1 frees the
+// chain's slots for the next call that writes this set; then warp 0 draws U while the
 // others reduce delta^T G over the rejected row, and they write y.  Every output is written
 // after griddep_wait.  Bound by the latency of one warp's evaluations (scan 4-5 us, U 4 us);
 // what does not depend on them runs beside them: with 64 threads, the noise before the scan's
@@ -140,19 +127,12 @@ __global__ void __launch_bounds__(NT) k_finish(VerifyArgs A) {
   // the next kernel (the next call's stream) may start now: it writes the other set of
   // partials, and a slot of this set only once this call has read it
   griddep_launch_dependents();
-  // a call's k_tiles CTA overwrites a slot once it reads back (acquire) the tag it found there
-  auto release_slots = [&](int g) {
-    if (!A.S.consumed) return;
-    const int64_t s0 = (int64_t)b * L * A.S.C;
-    const int n = g * A.S.C;
-    for (int k = lane; k < n; k += 32)
-      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(A.S.consumed + s0 + k), "r"(A.S.tag) : "memory");
-  };
   ScanOut so;
   OneWarp co;
   if (warp == 0) {
     float leta[2];
     scan_coins(A.S, b, leta);
+    if (A.S.fresh_set) griddep_wait();   // any tag may be in its slots
     ScanRegs R = scan_load(A.S, b);
     if (R.stale) {
       // a partial of this call is not visible yet (k_finish starts once every k_tiles
@@ -171,14 +151,14 @@ __global__ void __launch_bounds__(NT) k_finish(VerifyArgs A) {
     }
     if (lane == 0) gw_s = R.g;
     __syncwarp();
-    // warp 1 may release the slots (named barrier: this warp only arrives)
+    // warp 1 may free the slots (named barrier: this warp only arrives)
     asm volatile("bar.arrive 1, 64;" ::: "memory");
     so = scan_decide(A.S, b, R, leta, co);
     if (lane == 0) fs.cs = so.cs;
   } else {
     if (warp == 1) {
       asm volatile("bar.sync 1, 64;" ::: "memory");
-      release_slots(gw_s);
+      slots_free(A.S.tpart + 2 * ((int64_t)b * L * A.S.C), lane, 32, gw_s * A.S.C);
     }
     draw_noise<HOLD>(seed, b, sl, g_s);
   }
@@ -358,12 +338,12 @@ WsLayout ws_layout(int B, int L, int64_t d, int dtype) {
   size_t off = 0;
   w.part_off = off;
   const size_t slots = (size_t)B * L * w.C1;
-  w.cons_off = up(2 * sizeof(uint64_t) * slots);  // within a set
-  w.part_set_bytes = up(w.cons_off + sizeof(uint32_t) * slots);
+  // 4 bytes a slot are not used (see below)
+  w.part_set_bytes = up(up(2 * sizeof(uint64_t) * slots) + sizeof(uint32_t) * slots);
   off = up(off + 2 * w.part_set_bytes);
-  // Not used since finishing keeps its state on chip: a counter and a state per chain, and a
-  // sum per 1024 to 4096 elements of a row (about 1024 in all).  The size stays, so that
-  // sizes that callers have stored, and sdv_verify_noalloc's limit, mean the same calls.
+  // Not used since slots are freed in place and finishing keeps its state on chip: a tag per
+  // slot, a counter and a state per chain, and a sum per 1024 to 4096 elements of a row (about
+  // 1024 in all).  The size stays, so that sizes that callers have stored, and sdv_verify_noalloc's limit, mean the same calls.
   int64_t chunk = 1024;
   while (chunk < 4096 && (int64_t)B * ((d + chunk - 1) / chunk) > 1024) chunk *= 2;
   off = up(off + 4 * (size_t)B);
@@ -448,10 +428,9 @@ static cudaError_t launch_finish(const VerifyArgs& A, int B, bool vec4, cudaStre
   return launch_ex(k_finish<T, false, kFinishThreads>, (unsigned)B, kFinishThreads, smem, A, s);
 }
 
-// The tag of a call's k_tiles partials: a process-wide counter, never 0 (a zeroed
-// workspace holds tag 0), so consecutive calls on a workspace never share a tag (a
-// captured call keeps its tag at every replay of its graph, and replays of a graph run
-// one after another).
+// The tag of a call's k_tiles partials: a process-wide counter, never 0 (a free slot's),
+// so consecutive calls on a workspace never share a tag.  A captured call keeps its tag at
+// every replay of its graph; replays run one after another, and each leaves its slots free.
 static std::atomic<uint32_t> g_partial_tag{0u};
 static uint32_t next_partial_tag() {
   uint32_t t;
@@ -541,9 +520,7 @@ static int enqueue_verify(const void* x_draft, const void* mu_target, const void
   bool fresh = true;
   char* set = ws + w.part_off + (size_t)g_partial_sets.next(workspace, layout, &fresh) * w.part_set_bytes;
   S.fresh_set = fresh;
-  A.tpart = (uint64_t*)set;
-  S.tpart = A.tpart;
-  S.consumed = (uint32_t*)(set + w.cons_off);
+  S.tpart = (uint64_t*)set;
   S.tag = next_partial_tag();
   e = f32 ? launch_tiles<float>(A, B, L, w.vpt1, rows, s)
           : launch_tiles<__nv_bfloat16>(A, B, L, w.vpt1, rows, s);

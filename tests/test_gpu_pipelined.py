@@ -208,3 +208,57 @@ def test_pipelined_large_and_small_calls_in_turn(api):
     torch.cuda.synchronize()
     for i, sh in enumerate(order):
         _same(piped[i], _call(api, sets[sh], 1100 + i, "block", ws))
+
+
+# Calls that stream with k_tiles: more chains than k_chain takes, ragged windows, a cluster per
+# chain, and a pipelined call; (the last) more partials than the cluster stages on chip.
+STREAMED = [("pixel", 310, 4, 300, False, False), ("pixel", 320, 6, 1000, True, False),
+            ("latent", 24, 16, 20000, False, False), ("pixel", 40, 6, 1000, True, True),
+            ("latent", 1, 64, 830000, False, False)]
+
+
+def _clone(s):
+    return {k: v.clone() for k, v in s.items()}
+
+
+@pytest.mark.parametrize("kind,B,L,d,ragged,pipelined", STREAMED[:4])
+def test_replayed_calls_follow_their_inputs(api, kind, B, L, d, ragged, pipelined):
+    """A graph of one call (and one of three: each set once or twice), its window, sigma and
+    window lengths changed between replays: a replayed call's tag is the one it was captured
+    with, and its slots must not pass for this replay's (against plain calls)."""
+    sets = _sets(kind, 3, B, L, d, ragged)
+    dt = sets[0]["x"].dtype
+    for n in (1, 3):
+        ws = torch.zeros(api.workspace_bytes(B, L, d, dt), dtype=torch.uint8, device="cuda")
+        live = [_clone(sets[0]) for _ in range(n)]
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            _call(api, live[0], 1, "block", ws, pipelined=pipelined)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            outs = [_call(api, live[i], 40 + i, "block", ws, pipelined=pipelined) for i in range(n)]
+        for rep in range(5):
+            for i in range(n):
+                for k, v in live[i].items():
+                    v.copy_(sets[(rep + i) % 3][k])
+            torch.cuda.synchronize()
+            g.replay()
+            torch.cuda.synchronize()
+            for i in range(n):
+                s = sets[(rep + i) % 3]
+                fresh = torch.zeros_like(ws)
+                act = s["L_eff"] > 0 if ragged else None
+                _same(outs[i], _call(api, s, 40 + i, "block", fresh), act)
+
+
+@pytest.mark.parametrize("kind,B,L,d,ragged,pipelined", STREAMED)
+def test_a_finished_call_leaves_its_slots_free(api, kind, B, L, d, ragged, pipelined):
+    """No partial stays behind for a replay to take for its own: a workspace of zeros (every
+    slot free) holds zeros again after any number of calls."""
+    s = _sets(kind, 1, B, L, d, ragged)[0]
+    ws = torch.zeros(api.workspace_bytes(B, L, d, s["x"].dtype), dtype=torch.uint8, device="cuda")
+    for n in range(3):
+        _call(api, s, 5 + n, "block", ws, pipelined=pipelined)
+        torch.cuda.synchronize()
+        assert int(torch.count_nonzero(ws)) == 0
