@@ -535,7 +535,9 @@ static int launch_rounds_t(RoundsArgs A, cudaStream_t s) {
   A.pre = (int)std::min<size_t>((size_t)A.L, kAhead / row);
   const size_t smem = row * (size_t)(1 + A.pre);
   if (smem > 32 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_rounds<MAXC, NT, NG, VEC, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is shared by all host threads: that of this kernel's longest rows
+    constexpr size_t kMost = sizeof(float4) * NT * NG + kAhead;
+    const cudaError_t e = cudaFuncSetAttribute(k_rounds<MAXC, NT, NG, VEC, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMost);
     if (e != cudaSuccess) {
       set_last_cuda_error((int)e);
       cudaGetLastError();

@@ -799,11 +799,12 @@ struct GmmLaunch {
   int maxc;
 };
 
+// The kernels' limit of dynamic shared memory, which all host threads share: its largest value.
 template <int MAXC, bool VEC>
-static void gmm_set_smem(size_t bytes) {
-  cudaFuncSetAttribute(k_gmm_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_round_target<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  cudaFuncSetAttribute(k_em_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+static void gmm_set_smem() {
+  cudaFuncSetAttribute(k_gmm_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmmSmemCap);
+  cudaFuncSetAttribute(k_round_target<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmmSmemCap);
+  cudaFuncSetAttribute(k_em_rows<MAXC, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGmmSmemCap);
 }
 
 // rows_aligned: every state / output row the kernel touches starts on a 16-byte boundary
@@ -815,8 +816,8 @@ static GmmLaunch gmm_launch(int C, int64_t d, const void* means, bool rows_align
   g.vec = (d % 4 == 0) && (reinterpret_cast<uintptr_t>(means) % 16 == 0) && rows_aligned;
   g.maxc = C <= 8 ? 8 : 16;
   if (g.smem_bytes > 48 * 1024) {
-    if (g.maxc == 8) { gmm_set_smem<8, true>(g.smem_bytes); gmm_set_smem<8, false>(g.smem_bytes); }
-    else { gmm_set_smem<16, true>(g.smem_bytes); gmm_set_smem<16, false>(g.smem_bytes); }
+    if (g.maxc == 8) { gmm_set_smem<8, true>(); gmm_set_smem<8, false>(); }
+    else { gmm_set_smem<16, true>(); gmm_set_smem<16, false>(); }
   }
   return g;
 }
@@ -859,9 +860,12 @@ template <int MAXC, int NG, int T>
 static int launch_em_t(int B, int64_t d, const Sched& S, const Gmm& G, uint64_t seed, float* y, cudaStream_t s) {
   const int sms = sm_count();
   const int teams = T == 8 ? 1 : std::min(kEmMaxTeams, std::max(1, (B + sms - 1) / sms));
-  const size_t smem = sizeof(float4) * (size_t)(G.C + teams) * 32 * NG + sizeof(float) * (size_t)teams * MAXC;
+  constexpr auto bytes = [](int c, int n) { return sizeof(float4) * (size_t)(c + n) * 32 * NG + sizeof(float) * (size_t)n * MAXC; };
+  const size_t smem = bytes(G.C, teams);
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_em_chain<MAXC, NG, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit is shared by all host threads: its largest value
+    constexpr int kMost = (int)bytes(MAXC, T == 8 ? 1 : kEmMaxTeams);
+    const cudaError_t e = cudaFuncSetAttribute(k_em_chain<MAXC, NG, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
     if (e != cudaSuccess) {
       set_last_cuda_error((int)e);
       cudaGetLastError();

@@ -366,15 +366,17 @@ static int validate_window(const void* x, const void* mq, const void* mp, const 
   return SDV_OK;
 }
 
-// A launch through cudaLaunchKernelEx: dynamic shared memory (raising the kernel's limit
-// when it passes 48 KB) and programmatic stream serialisation (the kernels wait for the
-// work before them where they need it).
+// A launch through cudaLaunchKernelEx: dynamic shared memory (raising the kernel's limit when
+// it passes 48 KB, to what the longest rows take: all host threads share the limit, so that a
+// call must not set it to its own size) and programmatic stream serialisation (the kernels
+// wait for the work before them where they need it).
+constexpr size_t kLaunchSmemMax = sizeof(float4) * (size_t)kPipeMaxGroups;
 template <typename Kern>
 static cudaError_t launch_ex(Kern kern, unsigned grid, unsigned threads, size_t smem, const VerifyArgs& A,
                              cudaStream_t s) {
   // the kernels' static shared memory counts toward the 48 KB that need no permission
   if (smem > 40 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLaunchSmemMax);
     if (e != cudaSuccess) return e;
   }
   cudaLaunchConfig_t cfg = {};

@@ -475,3 +475,51 @@ def test_log_ratios_of_an_enormous_row(api):
     ell_o, dn_o = OV.log_ratios(inp["x_draft"], inp["mu_target"], inp["mu_draft"], inp["sigma"])
     assert abs(lr.item() - ell_o.item()) <= 1e-5 * max(1.0, abs(ell_o.item()))
     assert abs(dn.item() - dn_o.item()) <= 1e-5 * max(1.0, dn_o.item())
+
+
+def test_threads_with_calls_of_different_shared_memory(api):
+    """Host threads whose calls run one kernel with different amounts of dynamic shared
+    memory, each on its own stream and workspace: a kernel's limit is a property of the
+    device, so that no call may set it to its own size."""
+    import threading
+
+    def verify_of(d, n):
+        inp = W.make_verify_inputs("pixel", B=2, L=2, d=d)
+        t = [torch.from_numpy(inp[k]).cuda() for k in ("x_draft", "mu_target", "mu_draft", "sigma")]
+        ws = api.make_workspace(2, 2, d, torch.float32)
+        out = api.verify(*t, 1, "block", workspace=ws)
+        return n, lambda: api.verify(*t, 1, "block", workspace=ws, out=out, with_ratios=False, pipelined=True)
+
+    def target(C, d, K):
+        means = torch.zeros(C, d)
+        return api.GmmTarget(means, torch.full((C,), -float(np.log(C))), 1.0, K, 0.5)
+
+    def rounds_of(d, n):
+        tgt = target(8, d, 40)
+        return n, lambda: api.sampler_run(4, 8, tgt, 3, "block", "free", max_rounds=1)
+
+    def em_of(B, C, d, n):
+        tgt = target(C, d, 2)
+        return n, lambda: api.em_sample(B, tgt, 3)
+
+    for pair in ((verify_of(16384, 4000), verify_of(11000, 4000)), (rounds_of(1024, 400), rounds_of(1020, 400)),
+                 (em_of(1024, 8, 1024, 2000), em_of(1024, 7, 1024, 2000)),
+                 (em_of(8, 8, 2048, 2000), em_of(8, 7, 2048, 2000))):
+        errors = []
+
+        def work(n, call):
+            try:
+                with torch.cuda.stream(torch.cuda.Stream()):
+                    for _ in range(n):
+                        call()
+                    torch.cuda.current_stream().synchronize()
+            except Exception as e:      # the main thread reports it
+                errors.append(e)
+        torch.cuda.synchronize()
+        ts = [threading.Thread(target=work, args=p) for p in pair]
+        for t in ts:
+            t.start()
+        for t in ts:
+            t.join()
+        torch.cuda.synchronize()
+        assert not errors, errors[0]
