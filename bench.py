@@ -24,6 +24,7 @@ Prints ONE JSON line (rank 0):
 --impl reference times the CPU oracle alone (the reference arm of this build).
 """
 import argparse
+import ctypes
 import hashlib
 import json
 import math
@@ -152,68 +153,47 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
-# The phases of a call by its sizes: rows of more than this many groups of four elements have
-# their residual's sum and write counted apart; pipelined calls finish rows of up to
-# PIPE_MAX_GROUPS in k_finish (the library's kPipeMaxGroups).
-FUSED_MAX_GROUPS = 1024
-FINISH_MAX_GROUPS = 1024
-PIPE_MAX_GROUPS = 4096
-
-# From this many chains on, a call is counted as streaming and finishing.
-MANY_CHAIN_MIN = 512
+class _KernelNode(ctypes.Structure):
+    """CUDA_KERNEL_NODE_PARAMS_v2 of the driver API."""
+    _fields_ = ([("func", ctypes.c_void_p)]
+                + [(n, ctypes.c_uint) for n in ("grid_x", "grid_y", "grid_z", "block_x", "block_y", "block_z", "smem")]
+                + [(n, ctypes.c_void_p) for n in ("params", "extra", "kern", "ctx")])
 
 
-def many_chains(B):
-    return B >= MANY_CHAIN_MIN
+def kernel_name(symbol):
+    """The kernel's own name in the mangled symbol of one of this library's kernels."""
+    m = re.match(r"_ZN3sdv(\d+)", symbol)
+    return symbol[m.end():m.end() + int(m.group(1))] if m else symbol
 
 
-def pipelined_path(d, pipelined):
-    """Does the call take the pipelined path (every kernel launched to overlap its
-    predecessor)?  Every pipelined call does."""
-    return bool(pipelined)
+def kernels_of_call(stream, call):
+    """Kernels that one call launches, in order: those of a CUDA graph that captures it."""
+    import torch
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g, stream=stream):
+        call()
+    cu = ctypes.CDLL("libcuda.so.1")
 
-
-def wide_finish(B, d, pipelined=False):
-    """Rows of 1025-4096 groups of four finished by a 256-thread k_finish (pipelined
-    calls, or plain calls with fewer than MANY_CHAIN_MIN chains)."""
-    ng = (d + 3) // 4
-    return FINISH_MAX_GROUPS < ng <= PIPE_MAX_GROUPS and (pipelined or not many_chains(B))
-
-
-# Plain calls with fewer chains are counted as one phase.
-FUSED_MAX_CHAINS = 64
-
-
-def _two_kernels(B, d, pipelined):
-    return B >= FUSED_MAX_CHAINS or bool(pipelined) or wide_finish(B, d, pipelined)
-
-
-def long_rows(d, B=0, pipelined=False):
-    """Rows whose residual counts as two more phases (longer than one finishing CTA's noise
-    cache)."""
-    if wide_finish(B, d, pipelined):
-        return False
-    return (d + 3) // 4 > (FINISH_MAX_GROUPS if _two_kernels(B, d, pipelined) else FUSED_MAX_GROUPS)
-
-
-def launches_per_step(B, d, pipelined=False):
-    """Phases of a verification call by its sizes: the whole call, or streaming and finishing
-    (many chains, a pipelined call, or rows of 1025-4096 groups), plus the residual's sum and
-    write for long rows.  Several may share a kernel: kernels_of_step lists the launches."""
-    return (2 if _two_kernels(B, d, pipelined) else 1) + (2 if long_rows(d, B, pipelined) else 0)
-
-
-def kernels_of_step(B, d, pipelined=False, L=8, dt_name="f32"):
-    """Kernels one verification call launches, in order (sizes of the library's routing rule,
-    152 SMs; without its limits on clusters of CTAs and on shared memory)."""
-    if not pipelined and B <= 304:
-        es = 2 if dt_name == "bf16" else 4
-        vecs = -(-d * es // 16)
-        tiles = L * -(-vecs // (256 * max(1, min(2 if es == 2 else 4, -(-vecs // 256)))))
-        cl = max(1, min(8, tiles, 304 // B))
-        if 10 * B * cl >= 13 * 152 or 3 * L * d * es // cl <= 256 * 1024:
-            return ["k_chain"]
-    return ["k_tiles", "k_finish" if (d + 3) // 4 <= PIPE_MAX_GROUPS else "k_finish_long"]
+    def check(rc):
+        if rc != 0:
+            raise RuntimeError("CUDA driver error %d while reading a captured call" % rc)
+    graph, n = ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0)
+    check(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    check(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    names = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(-1), _KernelNode(), ctypes.c_char_p()
+        check(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value != 0:          # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        check(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        if p.func:
+            check(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)))
+        else:
+            check(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+        names.append(kernel_name(name.value.decode()))
+    return names
 
 
 def call_bytes(B, L, d, dtype):
@@ -555,6 +535,7 @@ def measure_verify(api, name, Bn, mode, steps, warmup, dev, rank, pg=None, clock
         clk = clocks.stop() if clocks else None
         return dict(name=name, ms_step=ms_step, clocks=clk)
 
+    kernels = kernels_of_call(stream, lambda: step(0))
     # the roofline's duration: 200 back-to-back calls in one graph, events at its ends only
     g200 = _graph_of_calls(stream, 200, step)
     _replay_ms(stream, [g200])
@@ -582,14 +563,14 @@ def measure_verify(api, name, Bn, mode, steps, warmup, dev, rank, pg=None, clock
     return dict(
         name=name, B=Bn, L=L, d=d, dtype=dt_name, n_sets=n_sets, set_bytes=set_bytes, l2=l2,
         ms_step=ms_step, ms_call=ms_call, ms_steady=ms_ss, steady_calls=200 * reps_ss,
-        value_per_rank=Bn * L / (ms_step * 1e-3), taus=taus, clocks=clk, host0=host0,
+        value_per_rank=Bn * L / (ms_step * 1e-3), kernels=kernels, taus=taus, clocks=clk, host0=host0,
         roofline={"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                   "frac": achieved / hbm_peak, "peak_kind": peak_kind,
-                  "kernel": "whole call (%s)" % ", ".join(kernels_of_step(Bn, d, pipelined, L, dt_name)),
+                  "kernel": "whole call (%s)" % ", ".join(kernels),
                   "duration": "per-call period of 200 back-to-back calls in one CUDA graph "
                               "(events at its two ends only)",
                   "duration_us": 1e3 * ms_call, "algorithmic_bytes": nbytes,
-                  "traffic": profile_traffic(name, Bn == cfg["B"], pipelined_path(d, pipelined))})
+                  "traffic": profile_traffic(name, Bn == cfg["B"], pipelined)})
 
 
 def measure_e2e(api, host0, Bn, L, d, dt_name, mode, dev, n_steps):
@@ -711,7 +692,7 @@ def main():
                 "hbm_gbs_step": r["roofline"]["algorithmic_bytes"] / (r["ms_step"] * 1e-3) / 1e9,
                 "roofline": r["roofline"], "mean_tau_block": r["taus"]["block"],
                 "mean_tau_sample": r["taus"]["sample"],
-                "gpu_launches": len(kernels_of_step(c["B"], c["d"], pipelined, c["L"], c["dtype"])) * args.steps}
+                "gpu_launches": len(r["kernels"]) * args.steps}
         subs["sampler"] = sampler_summary(api, dev)
 
     e2e_steps = max(20, min(400, args.steps))
@@ -742,7 +723,7 @@ def main():
                 "d2h_bytes_per_step": d2h,
                 "api": "api.HostStream (pinned [3,B,L,d] window in, accepted_len and y out, "
                        "copy of step i+1 overlapping step i)"},
-        "gpu_launches": len(kernels_of_step(Bn, d, pipelined, L, dt_name)) * args.steps,
+        "gpu_launches": len(head["kernels"]) * args.steps,
         "clocks": head["clocks"],
         "workloads": subs,
     }

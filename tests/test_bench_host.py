@@ -1,4 +1,4 @@
-"""bench.py's host-side accounting, checked on the CPU: launches per call, algorithmic
+"""bench.py's host-side accounting, checked on the CPU: kernel names, algorithmic
 bytes of a call, the shared workload name of both arms, and the lookup of a
 profile's traffic (only for the workload's full batch and a matching source hash)."""
 import os
@@ -13,20 +13,10 @@ class _Args:
         self.workload, self.mode = workload, mode
 
 
-def test_launches_per_pipelined_call():
-    assert bench.launches_per_step(256, 3072, True) == 2     # k_tiles + k_finish, overlapping
-    assert bench.launches_per_step(64, 16384, True) == 2     # k_finish with 256 threads
-    assert bench.launches_per_step(16, 196608, True) == 4    # + the long-row kernels, all overlapping
-    assert bench.kernels_of_step(256, 3072, True) == ["k_tiles", "k_finish"]
-
-
-def test_launches_per_call():
-    assert bench.launches_per_step(32, 3072) == 1       # fused kernel (fewer than 64 chains)
-    assert bench.launches_per_step(256, 3072) == 2      # k_tiles + k_finish
-    assert bench.launches_per_step(64, 16384) == 2      # plain: k_tiles + 256-thread k_finish
-    assert bench.launches_per_step(16, 196608) == 3     # + long-row dot and write
-    assert bench.launches_per_step(1024, 3072) == 2     # k_tiles + k_finish
-    assert bench.launches_per_step(1024, 16384) == 4    # k_finish caches up to 4096 elements
+def test_kernel_names():
+    assert bench.kernel_name("_ZN3sdv13k_finish_longIfLb1ELi1ELi512EEEvNS_10VerifyArgsEii") == "k_finish_long"
+    assert bench.kernel_name("_ZN3sdv7k_chainIfLi1ELi3ELb1ELi0EEEvNS_10VerifyArgsEi") == "k_chain"
+    assert bench.kernel_name("memset_kernel") == "memset_kernel"
 
 
 def test_algorithmic_bytes_of_a_call():
