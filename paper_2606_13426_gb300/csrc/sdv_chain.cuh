@@ -371,11 +371,11 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
   float2* tile_s = stage ? reinterpret_cast<float2*>(dyn_s) : nullptr;   // [L C]
   float4* g_s = dyn_s + (stage ? (L * C + 1) / 2 : 0);
   const RowSlice sl = cluster_slice(A.d, cl, rank);
-  uint64_t* const p = A.S.tpart + 2 * ((int64_t)b * L * C);
-  if (rank == 0 && (!stage || A.S.fresh_set)) griddep_wait();   // !stage: warp 0 reads the partials itself
+  if (rank == 0 && !stage) griddep_wait();                // warp 0 reads the partials itself
   if (rank == 0 && stage) {
+    uint64_t* const p = A.S.tpart + 2 * ((int64_t)b * L * C);
     auto fetch = [&](bool check) {
-      int stale = 0;
+      int stale = check && A.S.fresh_set;   // any tag may be in its slots
 #pragma unroll 4
       for (int t = threadIdx.x; t < g * C; t += NT) {
         const ulonglong2 v = slot_read(p + 2 * t);
@@ -388,14 +388,14 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
       griddep_wait();
       (void)fetch(false);
     }
-    slots_free(p, threadIdx.x, NT, g * C);
+    if (threadIdx.x >= 32) slots_free(p, (int)threadIdx.x - 32, NT - 32, g * C);   // warp 0 goes on to the coins
   }
   if (cl > 1) cluster_wait();
   finish_ahead<HOLD>(A, b, rank, sl, g_s, fs);
   finish_cluster<T, VEC4, HOLD, NT>(A, b, cl, rank, tile_s, sl, g_s, fs);
   if (rank == 0 && !stage) {
     __syncthreads();
-    slots_free(p, threadIdx.x, NT, g * C);
+    slots_free(A.S.tpart + 2 * ((int64_t)b * L * C), threadIdx.x, NT, g * C);
   }
 }
 

@@ -69,10 +69,9 @@ __device__ __forceinline__ void slot_store(uint64_t* p, uint32_t tag, float2 s) 
 }
 // Frees slots t0, t0 + dt, ... below n, once a barrier has shown that they are read.
 __device__ __forceinline__ void slots_free(uint64_t* p, int t0, int dt, int n) {
-  for (int t = t0; t < n; t += dt) {
-    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t), "l"(0ull) : "memory");
-    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t + 1), "l"(0ull) : "memory");
-  }
+  for (int t = t0; t < n; t += dt) asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t), "l"(0ull) : "memory");
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  for (int t = t0; t < n; t += dt) asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p + 2 * t + 1), "l"(0ull) : "memory");
 }
 
 // Per-lane values of one chain's window, held by one warp: step j in lane j & 31 of
