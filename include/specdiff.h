@@ -334,8 +334,8 @@ size_t sdv_sampler_workspace_bytes(int B, int L, int64_t d);
  * `max_rounds` rounds have run.  One round: gamma_k = min(L, K - k) draft steps, the
  * parallel target call at yhat_k .. yhat_{k+gamma_k}, sdv_verify_ex (residual or bonus
  * step), then k <- min(k + tau, K); a window that reaches K takes no bonus step.
- * Rows of up to 4096 elements whose chains are resident at once (a thread block each): one
- * kernel runs all rounds.  Else the rounds run as one CUDA graph launched on `stream`, a
+ * Rows of up to 4096 elements, of chains that are resident at once (a thread block each) or of
+ * a few times as many chains: one kernel runs all rounds.  Else the rounds run as one CUDA graph launched on `stream`, a
  * while node whose body is one round (draft, target call, verification, update), the round
  * counter and seed held in the workspace and the loop ended on the device once no chain is
  * active or max_rounds rounds ran; a few rounds in which no chain can finish are launched

@@ -53,8 +53,8 @@ __device__ __forceinline__ float warp_sums(float (&v)[N]) {
   return v[0];
 }
 
-// RB: rows per pass, 32 / MAXC for aligned rows of up to 1024 elements (every chain's CTA is
-// then resident at once, at 768 threads per SM), else one.
+// RB: rows per pass, 32 / MAXC for aligned rows of up to 1024 elements (at 768 threads per SM),
+// else one.
 template <int MAXC, int NT, int NG, bool VEC, int RB>
 __global__ void __launch_bounds__(NT, NG == 1 ? (RB == 1 ? 1024 : 768) / NT : 1) k_rounds(RoundsArgs A) {
   constexpr int NV = RB * MAXC;          // distances per pass

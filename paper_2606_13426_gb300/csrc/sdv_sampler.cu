@@ -1063,13 +1063,29 @@ static RoundsArgs rounds_args(const SamplerRun& R) {
   return A;
 }
 
-// Whether k_rounds runs the sampler: rows of up to kRoundMaxD elements, except aligned ones
-// of up to 1024 with more chains than are resident at once, which one kernel per phase of a
-// round serves better (d = 1024, L = 8: 456 chains 46 us a round against 61 in phases, 608
-// chains 88 against 74, 1024 chains 119 against 107).
+// Whether k_rounds runs the sampler (rows of up to kRoundMaxD elements) or one kernel per phase
+// of a round does.  k_rounds' time grows by whole waves of CTAs and with the threads' groups,
+// filled or not; the phases' with chains and elements, from a floor of five launches a round.
+//  - All chains in one wave, or means too large for the phases' shared memory: k_rounds (0.25 to
+//    0.99 of the phases' time over the sizes measured; but 1.06 for 152 chains of 2052 elements,
+//    L = 32, and 1.07 for 1824 of 256, L = 4).
+//  - Aligned rows of up to 1024 elements, more waves: phases (d = 1024, L = 8: 456 chains, one
+//    wave, 46 us a round against 61, 608 chains 88 against 74, 1024 chains 119 against 107).
+//  - Other rows: up to 7 (aligned) or 5 waves of full rows, fewer where a row leaves part of the
+//    groups empty, and, over 1024 elements, where the window outgrows the noise that is drawn
+//    ahead.  k_rounds over phases at L = 8 by waves: aligned 1028 1.2 at 7, 2048 0.90 at 7 and
+//    1.07 at 27, 2052 1.31 at 7; else 513 0.94 at 2 and 1.09 at 4, 901 0.82 at 2 and 1.01 at 8,
+//    1101 1.11 at 2 and 1.72 at 7, 2001 0.91 at 2 and 1.18 at 4, 3001 0.81 at 3.  At L = 16 and
+//    2 waves: 1028 1.09, 2048 0.74, 2052 1.11.
 static bool rounds_fit(const SamplerRun& R) {
   if (R.d > kRoundMaxD) return false;
-  return !R.gl.vec || R.d > 1024 || R.B <= sm_count() * (768 / round_threads(R.d));
+  const RoundShape s = round_shape(R.d, R.gl.vec);
+  const int64_t slots = (int64_t)sm_count() * s.per_sm, waves = (R.B + slots - 1) / slots;
+  if (waves <= 1 || !R.gl.smem) return true;
+  if (R.gl.vec && R.d <= 1024) return false;
+  const float full = (float)R.d / (float)(4 * s.threads * s.groups);
+  const float window = R.d > 1024 ? 8.0f / (float)std::max(8, R.L) : 1.0f;
+  return (float)waves <= (R.gl.vec ? 7.0f : 5.0f) * full * window;
 }
 
 static int launch_rounds(const SamplerRun& R, const RoundsArgs& A, cudaStream_t s) {

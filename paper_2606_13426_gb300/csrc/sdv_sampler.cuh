@@ -54,9 +54,18 @@ struct SamplerCtl {
 };
 
 constexpr int kRoundThreads = 256;
-// Threads of a chain's CTA for rows of up to 1024 elements (one group of four each).
-inline int round_threads(int64_t d) { return d <= 128 ? 32 : (d <= 256 ? 64 : (d <= 512 ? 128 : kRoundThreads)); }
 constexpr int64_t kRoundMaxD = 4 * 4 * kRoundThreads;   // NG <= 4
+// How k_rounds takes a row: a chain's threads, groups of four per thread, and the CTAs of an SM
+// by threads and registers (long windows of short rows can ask for more shared memory than
+// leaves place for as many).
+struct RoundShape {
+  int threads, groups, per_sm;
+};
+inline RoundShape round_shape(int64_t d, bool vec) {
+  if (d > 1024) return {kRoundThreads, vec && d <= 2048 ? 2 : 4, 1};
+  const int t = vec ? (d <= 128 ? 32 : (d <= 256 ? 64 : (d <= 512 ? 128 : kRoundThreads))) : (d <= 256 ? 64 : kRoundThreads);
+  return {t, 1, (vec ? 768 : 1024) / t};
+}
 
 struct RoundsArgs {
   float* y;       // [B, d] states

@@ -239,7 +239,10 @@ def test_first_rounds_other_shapes(api, d, C):
 @pytest.mark.parametrize("Bn,d,C,L", [(2, 3, 1, 4), (9, 128, 8, 5), (9, 129, 9, 5), (40, 256, 16, 4), (40, 257, 2, 33),
                                       (33, 513, 8, 64), (460, 600, 8, 4), (460, 516, 12, 4), (1830, 200, 8, 4),
                                       (12, 1026, 8, 6), (12, 2048, 9, 12), (12, 2052, 8, 4), (6, 4096, 8, 4),
-                                      (6, 4093, 3, 4), (6, 4100, 8, 4), (6, 4099, 12, 4)])
+                                      (6, 4093, 3, 4), (6, 4100, 8, 4), (6, 4099, 12, 4),
+                                      # several waves of chains, in the round kernel and, past them, in phases
+                                      (310, 1028, 8, 4), (470, 1028, 8, 4), (310, 1029, 8, 4), (310, 2052, 8, 16),
+                                      (310, 2601, 4, 4), (1220, 701, 8, 4), (620, 401, 8, 4)])
 @pytest.mark.parametrize("mode,drafter", [(OV.MODE_BLOCK, "frozen"), (OV.MODE_SAMPLE, "free")])
 def test_round_kernel_edges(api, Bn, d, C, L, mode, drafter):
     _first_rounds(api, mode, drafter, d, C, Bn=Bn, L=L, K=200, chains=np.unique(np.linspace(0, Bn - 1, 12).astype(int)))
