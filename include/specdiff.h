@@ -361,7 +361,8 @@ int sdv_sampler_run(int B, int L, int64_t d, const float *means, const float *lo
  * sdv_sampler_run, so that begin + R rounds + end gives the same results
  * as sdv_sampler_run with max_rounds = R while a chain is active; a round with no
  * active chain only advances the round counter); sdv_sampler_end synchronises
- * `stream` and returns the same outputs as sdv_sampler_run.  Every round must pass
+ * `stream` and returns the same outputs as sdv_sampler_run.  Rounds may also follow
+ * sdv_sampler_run itself, which leaves its state in the workspace.  Every round must pass
  * the arguments given to begin (and one mode and drafter throughout).  All three
  * return SDV_EINVAL / SDV_ENOWORKSPACE / SDV_EALIGN for bad arguments as
  * sdv_sampler_run does, before launching anything.

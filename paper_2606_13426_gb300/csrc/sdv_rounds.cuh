@@ -505,12 +505,17 @@ __global__ void __launch_bounds__(NT, NG == 1 ? (RB == 1 ? 1024 : 768) / NT : 1)
     for (int i = 0; i < NG; ++i) {
       store4f(yrow, tid + NT * i, y[i]);
       store4f(scrow, tid + NT * i, sc[i]);
+      if (A.y_out) store4f(A.y_out + (int64_t)b * d, tid + NT * i, y[i]);
     }
     if (tid == 0) {
+      const int nr = A.fresh ? lr : A.rounds[b] + lr, nt = A.fresh ? tsum : A.tsum[b] + tsum;
       A.kk[b] = k;
       A.gam[b] = g;
-      A.rounds[b] = A.fresh ? lr : A.rounds[b] + lr;
-      A.tsum[b] = A.fresh ? tsum : A.tsum[b] + tsum;
+      A.rounds[b] = nr;
+      A.tsum[b] = nt;
+      if (A.k_out) A.k_out[b] = k;
+      if (A.rounds_out) A.rounds_out[b] = nr;
+      if (A.tsum_out) A.tsum_out[b] = nt;
     }
   }
   if (tid == 0) {

@@ -1100,7 +1100,7 @@ static int read_results(const SamplerRun& R, float* y_out, int32_t* k_out, int32
       cudaStreamSynchronize(s) != cudaSuccess)
     return launch_check(), SDV_ECUDA;
   *rounds_out = r;
-  // outputs that the run wrote in place stay where they are
+  // outputs that the run wrote itself stay where they are
   auto copy = [&](void* out, const void* from, size_t bytes) {
     return out == nullptr || out == from || cudaMemcpyAsync(out, from, bytes, cudaMemcpyDeviceToDevice, s) == cudaSuccess;
   };
@@ -1173,15 +1173,16 @@ int sdv_sampler_run(int B, int L, int64_t d, const float* means, const float* lo
   if (rc != SDV_OK) return rc;
   cudaStream_t s = (cudaStream_t)stream;
   if (max_rounds > 0 && rounds_fit(R)) {
-    // one kernel from Y_0 to the outputs, which it writes in place where they are aligned
+    // one kernel from Y_0 to the outputs, which it writes itself where they are aligned; the
+    // workspace gets the state too, so that sdv_sampler_round can continue the run
     RoundsArgs A = rounds_args(R);
     A.fresh = 1;
     A.max_rounds = max_rounds;
     auto at = [](const void* p, size_t a) { return reinterpret_cast<uintptr_t>(p) % a == 0; };
-    if (at(y_out, R.gl.vec ? 16 : 4)) A.y = R.y = y_out;
-    if (k_out && at(k_out, 4)) A.kk = R.kk = k_out;
-    if (chain_rounds_out && at(chain_rounds_out, 4)) A.rounds = R.rounds = chain_rounds_out;
-    if (tau_sum_out && at(tau_sum_out, 4)) A.tsum = R.tsum = tau_sum_out;
+    if (at(y_out, R.gl.vec ? 16 : 4)) A.y_out = R.y = y_out;
+    if (k_out && at(k_out, 4)) A.k_out = R.kk = k_out;
+    if (chain_rounds_out && at(chain_rounds_out, 4)) A.rounds_out = R.rounds = chain_rounds_out;
+    if (tau_sum_out && at(tau_sum_out, 4)) A.tsum_out = R.tsum = tau_sum_out;
     if (cudaMemsetAsync(R.ctl, 0, sizeof(SamplerCtl), s) != cudaSuccess) return launch_check(), SDV_ECUDA;
     if ((rc = launch_rounds(R, A, s)) != SDV_OK) return rc;
     return read_results(R, y_out, k_out, chain_rounds_out, tau_sum_out, rounds_out, s);

@@ -72,6 +72,9 @@ struct RoundsArgs {
   float* sc;      // [B, d] cached scores
   float* rows;    // [B, L, dp] drafted states, dp = d rounded up to whole groups
   int32_t *kk, *gam, *rounds, *tsum;
+  // nullable: y, kk, rounds and tsum once more (sdv_sampler_run's outputs)
+  float* y_out;
+  int32_t *k_out, *rounds_out, *tsum_out;
   SamplerCtl* ctl;
   int B, L;
   int64_t d;

@@ -226,6 +226,30 @@ def test_host_driven_rounds_equal_graph_run(api, mode, drafter):
             assert torch.equal(g[key], h[key]), key
 
 
+# Runs of each form: one kernel (resident chains; several waves), rounds launched one after
+# another, a graph (chains that can finish), and one kernel with an unaligned row.
+@pytest.mark.parametrize("Bn,d,K,first", [(160, 64, 40, 2), (310, 1028, 100, 2), (620, 600, 100, 2), (620, 600, 12, 4),
+                                          (20, 37, 100, 2)])
+@pytest.mark.parametrize("drafter", ["free", "frozen"])
+def test_rounds_continue_a_run(api, Bn, d, K, first, drafter):
+    """A run leaves its state in the workspace: rounds after it give what a longer run does,
+    bit for bit."""
+    L, more = 4, 2
+    tgt = _target(api, _gmm(8, d, 11), K, 0.5)
+    whole = api.sampler_run(Bn, L, tgt, 77, "block", drafter, max_rounds=first + more)
+    ws = torch.zeros(api.B.sdv_sampler_workspace_bytes(Bn, L, d), dtype=torch.uint8, device="cuda")
+    part = api.sampler_run(Bn, L, tgt, 77, "block", drafter, max_rounds=first, workspace=ws)
+    st = torch.cuda.current_stream().cuda_stream
+    dr = {"free": api.B.SDV_DRAFTER_FREE, "frozen": api.B.SDV_DRAFTER_FROZEN}[drafter]
+    for _ in range(more):
+        api.B.sdv_sampler_round(Bn, L, d, *tgt.params(), 77, api.B.SDV_MODE_BLOCK, dr, ws.data_ptr(), ws.numel(), st)
+    r = api.B.sdv_sampler_end(Bn, L, d, ws.data_ptr(), ws.numel(), part["y"].data_ptr(), part["k"].data_ptr(),
+                              part["chain_rounds"].data_ptr(), part["tau_sum"].data_ptr(), st)
+    assert r == whole["rounds"]
+    for key in ("y", "k", "chain_rounds", "tau_sum"):
+        assert torch.equal(part[key], whole[key]), key
+
+
 # Row lengths and component counts that take the other target-call kernels: ragged d
 # and rows longer than 1024 elements (shared-memory means), 9..16 components.
 @pytest.mark.parametrize("d,C", [(37, 8), (1100, 8), (64, 12), (1024, 12), (1030, 12)])
