@@ -10,6 +10,7 @@ import functools
 import importlib.util
 import os
 import threading
+import warnings
 
 from .buildlib import lib_path, pycall_path
 
@@ -117,13 +118,18 @@ def load(path=None):
 
 def _bind_native(lib):
     """The calls of a serving loop through the compiled module (ctypes takes 4-5 us to convert
-    their 25 arguments); without it (built where Python's headers are missing) ctypes serves."""
+    their 25 arguments); without it (Python's headers were missing, or it does not load here)
+    ctypes serves."""
     path = pycall_path()
     if not os.path.exists(path):
         return
-    spec = importlib.util.spec_from_file_location("_sdvcall", path)
-    mod = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(mod)
+    try:
+        spec = importlib.util.spec_from_file_location("_sdvcall", path)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+    except ImportError as e:
+        warnings.warn("libspecdiff: calls go through ctypes (%s)" % e)
+        return
     for name, fn in (("sdv_verify_ex", mod.verify), ("sdv_verify_pipelined", mod.verify),
                      ("sdv_log_ratios", mod.ratios)):
         _fns[name] = functools.partial(fn, ctypes.cast(getattr(lib, name), ctypes.c_void_p).value)

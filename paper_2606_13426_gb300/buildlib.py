@@ -2,8 +2,8 @@
 
 Sources are compiled in parallel, one nvcc process per translation unit, and
 linked into ``paper_2606_13426_gb300/lib/libspecdiff.so``; the CPython module of the
-binding's frequent calls goes beside it.  A rebuild happens only
-when a source or header is newer than the library (or ``force=True``).
+binding's frequent calls goes beside it.  Each is rebuilt only when one of its sources or
+headers is newer (or ``force=True``).
 """
 import os
 import shutil
@@ -30,18 +30,36 @@ def lib_path():
 
 
 def pycall_path():
-    return os.path.join(LIBDIR, "_sdvcall.so")
+    """The module's file, named for this Python's ABI."""
+    return os.path.join(LIBDIR, "_sdvcall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
 
 
-def _build_pycall():
-    """The CPython module of sdv_pycall.c; left out where Python's headers are missing (the
-    binding then calls through ctypes)."""
+def _pycall_source():
+    return os.path.join(CSRC, "sdv_pycall.c")
+
+
+def _python_headers():
     inc = sysconfig.get_paths()["include"]
-    if not os.path.exists(os.path.join(inc, "Python.h")):
+    return inc if os.path.exists(os.path.join(inc, "Python.h")) else None
+
+
+def _newer_than(out, deps):
+    if not os.path.exists(out):
+        return False
+    t = os.path.getmtime(out)
+    return all(os.path.getmtime(p) <= t for p in deps)
+
+
+def _build_pycall(force=False):
+    """The CPython module of sdv_pycall.c, if it is not up to date; left out where Python's
+    headers or a C compiler are missing (the binding then calls through ctypes)."""
+    inc, out = _python_headers(), pycall_path()
+    cc = os.environ.get("CC") or shutil.which("gcc") or shutil.which("cc")
+    if inc is None or cc is None or not force and _newer_than(out, [_pycall_source(), os.path.join(INCLUDE, "specdiff.h")]):
         return
-    out = pycall_path()
-    cmd = [os.environ.get("CC") or shutil.which("gcc") or "cc", "-O2", "-shared", "-fPIC", "-I" + INCLUDE, "-I" + inc,
-           os.path.join(CSRC, "sdv_pycall.c"), "-o", out + ".tmp"]
+    os.makedirs(LIBDIR, exist_ok=True)
+    cmd = [cc, "-O2", "-shared", "-fPIC", "-I" + INCLUDE, "-I" + inc,
+           _pycall_source(), "-o", out + ".tmp"]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("compiling sdv_pycall.c failed:\n%s\n%s" % (" ".join(cmd), r.stderr))
@@ -60,23 +78,21 @@ def _sources():
 
 
 def _deps():
-    deps = _sources() + [os.path.join(CSRC, "sdv_pycall.c")]
+    deps = _sources()
     for d in (CSRC, INCLUDE):
         deps += [os.path.join(d, f) for f in os.listdir(d) if f.endswith((".h", ".cuh"))]
     return deps
 
 
 def up_to_date():
-    out = lib_path()
-    if not os.path.exists(out):
-        return False
-    t = os.path.getmtime(out)
-    return all(os.path.getmtime(p) <= t for p in _deps())
+    return _newer_than(lib_path(), _deps())
 
 
 def build(force=False, verbose=False):
-    """Compile every CUDA source for sm_103a and link libspecdiff.so; returns its path."""
+    """Compile every CUDA source for sm_103a and link libspecdiff.so, and the module of the
+    binding's frequent calls; returns the library's path."""
     out = lib_path()
+    _build_pycall(force)
     if not force and up_to_date():
         return out
     nvcc = _nvcc()
@@ -97,7 +113,6 @@ def build(force=False, verbose=False):
     srcs = _sources()
     with ThreadPoolExecutor(max_workers=max(1, len(srcs))) as ex:
         objs = list(ex.map(compile_one, srcs))
-    _build_pycall()
     tmp = out + ".tmp"
     cmd = [nvcc] + ARCH + ["-shared", "-o", tmp] + objs
     r = subprocess.run(cmd, capture_output=True, text=True)

@@ -128,3 +128,29 @@ def test_python_binding_raises_on_error(lib):
     with pytest.raises(B.SDVError) as ei:
         B.sdv_accept_scan(0, 0, 4, 4, 0, 0, 1, 1.0, 0, 0, None)
     assert ei.value.code == B.SDV_EINVAL
+
+
+def test_build_makes_a_missing_call_module(lib, tmp_path, monkeypatch):
+    """A tree that has the library but not the module of the frequent calls gets it."""
+    from paper_2606_13426_gb300 import buildlib
+    if buildlib._python_headers() is None:
+        pytest.skip("no Python headers")
+    before = os.path.getmtime(buildlib.lib_path())
+    path = str(tmp_path / os.path.basename(buildlib.pycall_path()))
+    monkeypatch.setattr(buildlib, "pycall_path", lambda: path)
+    buildlib.build()
+    assert os.path.exists(path) and os.path.getmtime(buildlib.lib_path()) == before
+    made = os.path.getmtime(path)
+    buildlib.build()
+    assert os.path.getmtime(path) == made
+
+
+def test_a_module_that_does_not_load_leaves_ctypes(lib, tmp_path, monkeypatch):
+    from paper_2606_13426_gb300 import binding
+    bad = tmp_path / "bad.so"
+    bad.write_bytes(b"not a module")
+    monkeypatch.setattr(binding, "pycall_path", lambda: str(bad))
+    monkeypatch.setattr(binding, "_fns", {n: getattr(lib, n) for n in binding.SIGNATURES})
+    with pytest.warns(UserWarning, match="ctypes"):
+        binding._bind_native(lib)
+    assert binding._fns["sdv_verify_ex"] is lib.sdv_verify_ex
