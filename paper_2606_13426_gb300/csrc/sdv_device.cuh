@@ -25,23 +25,11 @@
 //  - for s < -4, lambda(s) + s = 1/(x + 2/(x + 3/(x + ...))), x = -s, which is
 //    Laplace's continued fraction for the Mills ratio with its first term
 //    cancelled analytically.
-#pragma once
-
-// Linkage of the special-function helpers (see above); a translation unit may
-// define SDV_HELPER before including this header.
-#ifndef SDV_HELPER
-#define SDV_HELPER __noinline__
-#endif
-// Unrolling of the quadrature's node pairs.  The code runs on one warp per chain, mostly
+// The quadratures' node pairs are not unrolled.  The code runs on one warp per chain, mostly
 // from a cold instruction cache: rolled, a pair's two nodes still overlap, and the smaller
-// code (gdiff 19 KB unrolled, of 130 KB in a finishing kernel) measured faster (pixel
-// batch 25.1 -> 23.9 us, tiny call 13.3 -> 12.7).
-#ifndef SDV_GL_UNROLL
-#define SDV_GL_UNROLL 1
-#endif
-namespace sdv {
-constexpr int kGLUnroll = SDV_GL_UNROLL;
-}
+// code (gdiff 19 KB unrolled, of 130 KB in a finishing kernel) measured faster (pixel batch
+// 25.1 -> 23.9 us, tiny call 13.3 -> 12.7).
+#pragma once
 
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -125,7 +113,7 @@ __device__ __forceinline__ float4 normals4(uint64_t seed, uint32_t b, uint32_t b
 }
 
 // normals4 as one shared copy, for the residual paths that run once per chain.
-static __device__ SDV_HELPER float4 normals4_f(uint64_t seed, uint32_t b, uint32_t blk, uint32_t stream,
+static __device__ __noinline__ float4 normals4_f(uint64_t seed, uint32_t b, uint32_t blk, uint32_t stream,
                                                uint32_t sub) {
   return normals4(seed, b, blk, stream, sub);
 }
@@ -200,10 +188,10 @@ __device__ __forceinline__ float2 log_ndtr_g(float a) {
 }
 
 // log Phi(a).
-static __device__ SDV_HELPER float log_ndtr(float a) { return log_ndtr_g(a).x; }
+static __device__ __noinline__ float log_ndtr(float a) { return log_ndtr_g(a).x; }
 
 // g(a) = log Phi(a) + a^2/2 (moderate for a <= 0).
-static __device__ SDV_HELPER float gfun(float a) { return log_ndtr_g(a).y; }
+static __device__ __noinline__ float gfun(float a) { return log_ndtr_g(a).y; }
 
 // g'(s) = lambda(s) + s > 0 in its two forms.  For s < -4 (x = -s) Laplace's
 // continued fraction for the Mills ratio with its first term cancelled,
@@ -285,7 +273,7 @@ __device__ __forceinline__ float gdiff_direct(float hi, float h) {
 }
 
 template <typename Coop>
-static __device__ SDV_HELPER float gdiff(float hi, float h, Coop& co) {
+static __device__ __noinline__ float gdiff(float hi, float h, Coop& co) {
   const unsigned act = __activemask();
   const bool careful = ((h < 0.5f) || (hi < -2.0f)) && (h <= fmaxf(2.0f, 0.5f * fabsf(hi)));
   const bool any_quad = __any_sync(act, careful), any_direct = __any_sync(act, !careful);
@@ -305,7 +293,7 @@ static __device__ SDV_HELPER float gdiff(float hi, float h, Coop& co) {
     if (any_direct) direct = co.at(4);
   } else {
     if (any_quad) {
-#pragma unroll kGLUnroll
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) acc += gdiff_pair(i, m, r, need_ex, need_cf);
     }
     if (any_direct) direct = gdiff_direct(hi, h);
@@ -335,7 +323,7 @@ __device__ __forceinline__ float logaddexp(float a, float b) {
 }
 
 // log(Phi(b) - Phi(a)) for a < b.
-static __device__ SDV_HELPER float log_ndtr_interval(float a, float b) {
+static __device__ __noinline__ float log_ndtr_interval(float a, float b) {
   if (b <= 0.0f) return log_ndtr(b) + log1mexp(log_ndtr(a) - log_ndtr(b));
   if (a >= 0.0f) return log_ndtr(-a) + log1mexp(log_ndtr(-b) - log_ndtr(-a));
   return log1pf(-(expf(log_ndtr(a)) + expf(log_ndtr(-b))));
@@ -364,7 +352,7 @@ struct UParams {
 };
 
 template <typename Coop>
-static __device__ SDV_HELPER UParams usample_setup(float D, float la, Coop& co) {
+static __device__ __noinline__ UParams usample_setup(float D, float la, Coop& co) {
   UParams P;
   P.D = D;
   P.la = la;
@@ -385,7 +373,7 @@ static __device__ SDV_HELPER UParams usample_setup(float D, float la, Coop& co) 
 // The first bracket is g(u) - g(a+) + t (a+ + u)/2 for a+ <= 0 (no term larger than
 // the result grows with |a+|) and a plain difference of log Phi otherwise.
 template <typename Coop>
-static __device__ SDV_HELPER float usample_log_psi(float t, const UParams& P, Coop& co) {
+static __device__ __noinline__ float usample_log_psi(float t, const UParams& P, Coop& co) {
   const float u = P.ap - t;
   const float x = -gdiff(u, P.D, co) - P.D * t;     // log(Phi(u - D) / (alpha Phi(u)))
   const float2 lg = log_ndtr_g(u);
@@ -403,7 +391,7 @@ __device__ __forceinline__ float usample_near_pair(int i, float r, const UParams
 }
 
 template <typename Coop>
-static __device__ SDV_HELPER float usample_log_1mpsi(float t, const UParams& P, Coop& co) {
+static __device__ __noinline__ float usample_log_1mpsi(float t, const UParams& P, Coop& co) {
   const unsigned act = __activemask();
   const bool near = P.D * t <= 1.0f && -P.am * t <= 4.0f;
   const bool any_near = __any_sync(act, near), any_far = __any_sync(act, !near);
@@ -426,7 +414,7 @@ static __device__ SDV_HELPER float usample_log_1mpsi(float t, const UParams& P, 
     }
   } else {
     if (any_near) {
-#pragma unroll kGLUnroll
+#pragma unroll 1
       for (int i = 0; i < 4; ++i) acc += usample_near_pair(i, r, P);
     }
     if (any_far) {

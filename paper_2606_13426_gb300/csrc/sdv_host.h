@@ -78,7 +78,6 @@ struct ScanArgs {
   float inv_omega2;
   int residual_kind;
   bool has_bonus;
-  bool ratios_only;
   float* ell_out;
   float* dn_out;
   int32_t* accepted_len;
@@ -86,7 +85,6 @@ struct ScanArgs {
   float* la_res_out;
   uint32_t* status_out;
   float* aux_out;
-  bool draw_u;  // draw the residual U (the whole verify step) or stop at tau
 };
 
 // Arguments of the kernels that stream a window or finish its chains.

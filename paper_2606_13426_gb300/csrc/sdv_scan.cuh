@@ -167,7 +167,6 @@ __device__ __forceinline__ void scan_write_steps(const ScanArgs& A, int b, const
 // The per-chain outputs known after the acceptance rule (accepted length, tau, log
 // alpha_res), by one thread.
 __device__ __forceinline__ void scan_write_chain(const ScanArgs& A, int b, const ChainState& cs) {
-  if (A.ratios_only) return;
   if (A.accepted_len) A.accepted_len[b] = cs.tau > 0 ? cs.tau - 1 : 0;
   if (A.tau_out) A.tau_out[b] = cs.tau;
   if (A.la_res_out && cs.kind != kKindInactive) A.la_res_out[b] = cs.la_res;
@@ -198,7 +197,7 @@ static __device__ ScanOut scan_decide(const ScanArgs& A, int b, const ScanRegs& 
   const int g = R.g;
   ScanOut out;
   out.have_P = false;
-  if (g <= 0 || A.ratios_only) {
+  if (g <= 0) {
     out.cs = inactive_state();
     return out;
   }

@@ -167,13 +167,11 @@ __global__ void __launch_bounds__(NT) k_finish(VerifyArgs A) {
   float coef = 0.f;
   if (cs.kind == kKindResid) {
     if (warp == 0) {
-      if (A.S.draw_u) {
-        const uint32_t wbits = philox_block(seed, (uint32_t)b, 0u, kStreamUSample, 0u).x;
-        uint32_t st = cs.status;
-        const UParams Q = so.have_P ? so.P : usample_setup(cs.dnorm, fminf(cs.la_res, 0.f), co);
-        cs.U = usample_warp(Q, wbits, &st, co);
-        cs.status = st;
-      }
+      const uint32_t wbits = philox_block(seed, (uint32_t)b, 0u, kStreamUSample, 0u).x;
+      uint32_t st = cs.status;
+      const UParams Q = so.have_P ? so.P : usample_setup(cs.dnorm, fminf(cs.la_res, 0.f), co);
+      cs.U = usample_warp(Q, wbits, &st, co);
+      cs.status = st;
       if (lane == 0) u_s = cs.U;
     } else {
       float dot = slice_dot<T, VEC4, HOLD>((const T*)A.mq, (const T*)A.mp, L, A.d, seed, b, cs, sl, rg, g_s);
@@ -463,7 +461,7 @@ static int enqueue_verify(const void* x_draft, const void* mu_target, const void
   S.C = w.C1; S.sigma = sigma; S.sstride = sigma_stride_b;
   S.B = B; S.L = L; S.L_eff = L_eff; S.seed = seed; S.seed_dev = seed_dev; S.mode = mode;
   S.inv_omega2 = 1.0f / (omega * omega); S.residual_kind = residual_kind;
-  S.has_bonus = mu_target_bonus != nullptr; S.ratios_only = ratios_only; S.draw_u = true;
+  S.has_bonus = mu_target_bonus != nullptr;
   S.ell_out = log_ratio_out; S.dn_out = delta_norm_out; S.accepted_len = accepted_len;
   S.status_out = status_out; S.aux_out = chain_aux_out;
 
@@ -666,7 +664,7 @@ int sdv_accept_scan(const float* log_ratio, const float* delta_norm, int B, int 
   ScanArgs A{};
   A.ell_in = log_ratio; A.dn_in = delta_norm; A.B = B; A.L = L; A.L_eff = L_eff;
   A.seed = seed; A.mode = mode; A.inv_omega2 = 1.0f / (omega * omega);
-  A.tau_out = tau_out; A.la_res_out = log_alpha_res_out; A.draw_u = false;
+  A.tau_out = tau_out; A.la_res_out = log_alpha_res_out;
   k_scan<<<(B + kK2Threads / 32 - 1) / (kK2Threads / 32), kK2Threads, 0, (cudaStream_t)stream>>>(A);
   return check_launch();
 }
