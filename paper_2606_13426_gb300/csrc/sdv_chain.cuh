@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(kK1Threads, kChainPerSm) k_chain(VerifyArgs A,
 
 // Threads of k_finish_long: 512 where every CTA has an SM to itself, else 256.
 constexpr int kLongThreads = 512, kLongThreadsMany = 256;
+constexpr int64_t kLongPairGroups = 8192;   // see launch_finish_long
 
 // The end of a call whose window k_tiles streams, for rows too long for one finishing CTA
 // (k_finish): a cluster per chain.  Its first CTA reads the chain's partials with all its
@@ -615,7 +616,12 @@ cudaError_t launch_finish_long(const VerifyArgs& A, int B, int L, bool vec4, cud
   // noise, four CTAs of 256 threads, two to an SM, so that the last wave of them is short; or
   // eight, where only those hold the noise.  (88 chains of one step of 96919 bf16 elements: 66 us
   // with eight, 68 with four, 124 with one of 512 threads; 150 x 1 x 50000 fp32 56 with four, 69
-  // with one; but 56 x 17 x 63432 140 with two of 512 threads, 168 with four of 256.)
+  // with one; but 56 x 17 x 63432 140 with two of 512 threads, 168 with four of 256.)  Two for at
+  // least a chain per SM of rows up to kLongPairGroups groups: every CTA of a chain holds its place
+  // through the chain's scan and U-draw, and there are more CTAs than places.  (Two against four:
+  // 512 chains of one step of 16388 fp32 elements 66 and 84 us, 505 x 1 x 30000 101 and 112, 152 x
+  // 1 x 30000 39 and 40; but 100 x 1 x 30000 36 and 30, 512 x 1 x 36000 133 and 129, 250 x 1 x
+  // 50000 106 and 88.)
   size_t tiles = 16 * (((size_t)L * A.S.C + 1) / 2);
   const auto noise = [&](int c) { return sizeof(float4) * (size_t)(((A.d + 3) / 4 + c - 1) / c); };
   const auto fits = [&](int c, size_t most) { return (tiles <= kFinishSmemMax / 2 ? tiles : 0) + noise(c) <= most; };
@@ -624,7 +630,8 @@ cudaError_t launch_finish_long(const VerifyArgs& A, int B, int L, bool vec4, cud
   if (cl > 1 && (fits(cl, kFinishSmemMax) || !fits(8, kChainSmemMax)))
     return vec4 ? launch_long_t<T, true, kLongThreads>(A, B, cl, tiles, noise(cl), s)
                 : launch_long_t<T, false, kLongThreads>(A, B, cl, tiles, noise(cl), s);
-  cl = fits(4, kChainSmemMax) || !fits(8, kChainSmemMax) ? 4 : 8;
+  if (B >= sm_count() && (A.d + 3) / 4 <= kLongPairGroups && fits(2, kChainSmemMax)) cl = 2;
+  else cl = fits(4, kChainSmemMax) || !fits(8, kChainSmemMax) ? 4 : 8;
   return vec4 ? launch_long_t<T, true, kLongThreadsMany>(A, B, cl, tiles, noise(cl), s)
               : launch_long_t<T, false, kLongThreadsMany>(A, B, cl, tiles, noise(cl), s);
 }

@@ -432,6 +432,8 @@ def test_one_kernel_calls(api, kind, B, L, d, mode):
                                                ("pixel", 160, 2, 60000, [0, 1, 80, 159]),
                                                ("latent", 88, 1, 60003, [0, 40, 87]),
                                                ("pixel", 40, 1, 120001, [0, 39]),
+                                               ("pixel", 160, 2, 32768, [0, 80, 159]), ("latent", 153, 3, 30001, [0, 152]),
+                                               ("pixel", 160, 1, 32772, [0, 159]),
                                                ("pixel", 520, 1, 16400, [0, 5, 519])])
 def test_long_rows(api, kind, B, L, d, sample, pipelined):
     _path_case(api, kind, B, L, d, chains=sample, pipelined=pipelined)
