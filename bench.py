@@ -83,11 +83,13 @@ def peaks():
     return 6800.0, "fallback"
 
 
-def kernel_sources_digest():
-    """sha256 over the sources that define the verify kernels (in a fixed order)."""
+def kernel_sources_digest(kernels=("k_tiles", "k_finish")):
+    """sha256 over the sources that define these kernels (in a fixed order)."""
+    files = ["sdv_verify.cu", "sdv_device.cuh", "sdv_host.h", "sdv_scan.cuh", "sdv_tiles.cuh", "sdv_finish.cuh"]
+    if not set(kernels) <= {"k_tiles", "k_finish"}:
+        files.append("sdv_chain.cuh")
     h = hashlib.sha256()
-    for f in ("sdv_verify.cu", "sdv_device.cuh", "sdv_host.h", "sdv_scan.cuh", "sdv_tiles.cuh", "sdv_finish.cuh",
-              "sdv_chain.cuh"):
+    for f in files:
         with open(os.path.join(ROOT, "paper_2606_13426_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -95,17 +97,19 @@ def kernel_sources_digest():
 
 def profile_traffic(workload, full_size, pipelined=True):
     """DRAM bytes per call (all of the call's kernels) on this workload from its committed
-    ncu summary (profiles/verify_<workload>_<pipelined|plain>.md), if the kernel sources
-    are unchanged since the capture and the batch is the workload's full one (else None)."""
+    ncu summary (profiles/verify_<workload>_<pipelined|plain>.md), if the sources of the
+    kernels that it lists are unchanged since the capture and the batch is the workload's full
+    one (else None)."""
     path = os.path.join(ROOT, "profiles", "verify_%s_%s.md" % (workload, "pipelined" if pipelined else "plain"))
     if not full_size or not os.path.exists(path):
         return None
     txt = open(path).read()
     m = re.search(r"traffic_bytes_per_call:\s*([0-9.eE+]+)", txt)
     h = re.search(r"kernel_source_sha256:\s*([0-9a-f]+)", txt)
-    if not m or not h:
+    k = re.search(r"profiled_kernels:\s*(.+)", txt)
+    if not m or not h or not k:
         return None
-    return float(m.group(1)) if h.group(1) == kernel_sources_digest() else None
+    return float(m.group(1)) if h.group(1) == kernel_sources_digest(re.split(r"[,\s]+", k.group(1).strip())) else None
 
 
 class ClockSampler:

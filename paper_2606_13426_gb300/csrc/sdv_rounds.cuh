@@ -24,8 +24,8 @@ namespace sdv {
 // only), the larger part of a round's instructions.  With few chains a round is bound by that
 // chain's latency (d = 1024, L = 8, up to one chain per SM: 21 us a round, 40 us with five
 // kernels a round in a graph and the windows in HBM); with many by the supply of instructions
-// (62 thousand warp instructions a chain and round, of which 35 % draw noise; 40 % of the
-// issue slots used), see rounds_fit.
+// (65 thousand warp instructions a chain and round; 456 chains use 60 % of the issue slots, the
+// rest goes to barriers and instruction fetches), see rounds_fit.
 // Sums over the warp of N values per lane (N = 2, 4, .. 32): lane l returns the sum of
 // value l / (32 / N), added over lanes in the order of an xor butterfly 16, 8, 4, 2, 1.
 template <int N>

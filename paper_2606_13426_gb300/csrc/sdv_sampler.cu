@@ -631,10 +631,11 @@ k_sampler_init(int B, int L, int64_t d, int K, uint64_t seed, float* y, int32_t*
 // warps share out the components (squared distances, pass 1), then the groups (score,
 // mean and noise, pass 2), and exchange the logits and the new state through shared
 // memory.  The sums have the order of gmm_rows_warp, so that both give the same states.
-// It is bound by instruction issue (of about 315 instructions per group of four and step,
-// 190 draw its noise); one launch per step with the state in HBM took 13.1 us a step at
-// B = 1024, d = 1024, C = 8, this kernel 4.7 us with T = 4 (T = 2: 5.5, too few warps; 8:
-// 5.4, seven eighths of the softmax repeated and two waves of CTAs).
+// It is bound by instruction issue: 77 % of the issue slots, 567 instructions of a warp per 32
+// groups of four and step, waiting warps mostly ready but not selected.  One launch per step
+// with the state in HBM took 13.1 us a step at B = 1024, d = 1024, C = 8, this kernel 4.7 us
+// with T = 4 (T = 2: 5.5, too few warps; 8: 5.4, seven eighths of the softmax repeated and two
+// waves of CTAs).
 constexpr int kEmMaxTeams = 7;   // chains per CTA: 152 SMs x 7 hold 1024 chains in one wave
 
 template <int MAXC, int NG, int T>
