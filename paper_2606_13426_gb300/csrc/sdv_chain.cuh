@@ -202,6 +202,8 @@ __device__ __forceinline__ void finish_ahead(const VerifyArgs& A, int b, int ran
   }
 }
 
+constexpr int kMaxScanners = 5;   // warps that share the scan's evaluations
+
 // From the chain's tile sums (tile_s of the cluster's first CTA) to its outputs.  g > 0.
 template <typename T, bool VEC4, int HOLD, int NT>
 __device__ __forceinline__ void finish_cluster(const VerifyArgs& A, int b, int cl, int rank, const float2* tile_s,
@@ -214,7 +216,7 @@ __device__ __forceinline__ void finish_cluster(const VerifyArgs& A, int b, int c
   // where CTAs have an SM to themselves, three where two share one and the rows wait in
   // registers (the others reduce delta^T G beside them), else its first warp alone.
   constexpr bool kAll = HOLD == kHoldAll;
-  const int scanners = gridDim.x <= (unsigned)A.sms ? 5 : (kAll ? 3 : 1);
+  const int scanners = gridDim.x <= (unsigned)A.sms ? kMaxScanners : (kAll ? 3 : 1);
   CtaWarps co{fs.coop, 0, scanners};
   RowRegs<own_groups(HOLD)> rg;
   ScanRegs R;
@@ -389,7 +391,9 @@ __global__ void __launch_bounds__(NT) k_finish_long(VerifyArgs A, int cl, int st
       griddep_wait();
       (void)fetch(false);
     }
-    if (threadIdx.x >= 32) slots_free(p, (int)threadIdx.x - 32, NT - 32, g * C);   // warp 0 goes on to the coins
+    // by the warps that the scan does not wait for
+    constexpr int kFirst = 32 * kMaxScanners;
+    if (threadIdx.x >= kFirst) slots_free(p, (int)threadIdx.x - kFirst, NT - kFirst, g * C);
   }
   if (cl > 1) cluster_wait();
   finish_ahead<HOLD>(A, b, rank, sl, g_s, fs);
