@@ -166,10 +166,11 @@ int sdv_verify_ex(const void *x_draft, const void *mu_target, const void *mu_dra
  * earlier work on `stream` that may still be running: the previous kernel, and the
  * earlier calls of a run of pipelined calls (the window is read while they finish).
  * The workspace needs no preparation: its two sets of tile partials are used
- * alternately by consecutive calls, each partial stored with a tag of its call; a
- * stream overwrites a slot only after the call that wrote it has read it (else it
+ * alternately by consecutive calls, each partial stored with a tag of its call and
+ * cleared when it has been read; a stream stores only into a clear slot (else it
  * waits for the previous kernel), and the finishing kernel waits for the whole stream
- * of its call when it reads a partial without its call's tag.
+ * of its call when it reads a partial without its call's tag.  The first calls after
+ * a change of (B, L, d) or of workspace wait for the call before them.
  * Outputs are written only after the previous call on `stream` has written its own,
  * so consecutive calls may share output buffers.  Same
  * arguments, return codes and ownership as sdv_verify_ex; the workspace must not be
@@ -206,9 +207,9 @@ int sdv_verify_pipelined(const void *x_draft, const void *mu_target, const void 
  *     device code there; make that first call before any stream capture on the
  *     device.
  *   - Every call on a device shares the one array, which keeps the previous call's
- *     contents: the counters that must start at zero are cleared by each call on its
- *     own stream, but calls that overlap on the GPU (other streams, other host
- *     threads, same device) race on the array.  Serialise them, e.g. on one stream.
+ *     contents: no call needs it prepared, but calls that overlap on the GPU (other
+ *     streams, other host threads, same device) race on the array.  Serialise them,
+ *     e.g. on one stream.
  */
 #define SDV_NOALLOC_SCRATCH_BYTES (1u << 22)
 int sdv_verify_noalloc(const void *x_draft, const void *mu_target, const void *mu_draft,

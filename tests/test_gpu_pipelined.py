@@ -3,12 +3,12 @@ on one stream (each call streams its window while the previous call's chains fin
 
 A pipelined call streams with the same tile reduction as a plain call, so its log
 ratios, accepted lengths and status bits equal a plain call's bit for bit; it finishes
-every chain with k_finish (the one-warp U-sampler, a 64-thread residual writer), so its
+every chain with k_finish or k_finish_long, which add up e^T G over other threads, so its
 U and states agree with a plain call's within the parity tolerances (U: 5e-6 + 3e-7|U|;
 states: 1e-5 absolute for fp32, 2e-2 for bf16), and one run is compared with the oracle
 directly.  Checked with separate outputs per call, with outputs shared by all calls
-(written in call order), under CUDA-graph capture, and with one workspace of arbitrary
-contents reused by calls of changing sizes."""
+(written in call order), under CUDA-graph capture, with inputs that change between replays, and
+with one workspace of arbitrary contents reused by calls of changing sizes."""
 import numpy as np
 import pytest
 import torch
@@ -150,9 +150,9 @@ def test_pipelined_calls_in_a_cuda_graph(api):
 
 
 def test_pipelined_long_rows(api):
-    """Rows longer than 16384 elements: k_tiles + k_finish without the residual, then the
-    long-row residual kernels, all four launched to overlap their predecessors (the
-    residual kernels sit resident, few and long, while the next call streams).  Against
+    """Rows longer than 16384 elements: k_tiles, then k_finish_long with a cluster per chain,
+    both launched to overlap their predecessors (the clusters sit resident, few and long,
+    while the next call streams).  Against
     plain calls on the same inputs (ratios, tau and status exact; U and states within
     the parity tolerance), with separate outputs, and the last call against the oracle."""
     B, L, d = 3, 4, 16388
@@ -169,8 +169,7 @@ def test_pipelined_long_rows(api):
 
 
 def test_pipelined_long_rows_many_chains(api):
-    """Many chains with long rows: the residual kernels keep one chunk per chain at least
-    (more chains than their CTA budget)."""
+    """Many chains with long rows: more clusters of k_finish_long than are resident at once."""
     B, L, d = 520, 2, 16388
     sets = _sets("pixel", 1, B, L, d, False)
     ws = torch.zeros(api.workspace_bytes(B, L, d, torch.float32), dtype=torch.uint8, device="cuda")
